@@ -14,8 +14,9 @@
 //
 // Roles (256 threads, one 128 x BN output tile per CTA, BN <= 128; two CTAs
 // fit one SM, whose tensor core then runs both CTAs' MMAs side by side):
-//   warp 0   one lane issues the TMA loads of a stage after the stage's
-//            "empty" barrier fired, with the byte count on its "full" barrier
+//   warp 0   issues the TMA loads of a stage (one elected lane) after the
+//            stage's "empty" barrier fired, with the byte count on its "full"
+//            barrier
 //   warp 1   waits "full", issues four tcgen05.mma (K = 16 each) and commits
 //            them to the stage's "empty" barrier; after the last stage it
 //            commits to the "accumulator ready" barrier
@@ -84,6 +85,7 @@ __device__ __forceinline__ bool mbar_try_wait(uint64_t *bar, uint32_t parity) {
 }
 
 __device__ __forceinline__ bool mbar_wait(uint64_t *bar, uint32_t parity) {
+  if (mbar_try_wait(bar, parity)) return true;
   const long long t0 = clock64();
   while (!mbar_try_wait(bar, parity)) {
     if (clock64() - t0 > kWaitCycles) return false;
@@ -138,20 +140,46 @@ __device__ __forceinline__ uint32_t instr_desc(int M, int N, bool a_mn, bool b_m
          ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
 }
 
-__device__ __forceinline__ void mma_bf16(uint32_t d_tmem, uint64_t a, uint64_t b, uint32_t idesc,
-                                         uint32_t accumulate) {
+// One lane of a converged warp (the same one every time).
+__device__ __forceinline__ bool elect_one() {
+  uint32_t p;
   asm volatile(
       "{\n\t.reg .pred p;\n\t"
-      "setp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(d_tmem),
-      "l"(a), "l"(b), "r"(idesc), "r"(accumulate)
+      "elect.sync _|p, 0xffffffff;\n\t"
+      "selp.u32 %0, 1, 0, p;\n\t}"
+      : "=r"(p));
+  return p != 0;
+}
+
+// One MMA, issued by one elected lane of the calling (converged) warp.  The
+// election sits around the instruction and not around the loop, so that the
+// loop stays warp-uniform and the operands (the descriptors' low and high
+// words) are computed in uniform registers, where the instruction reads them.
+// Issue rate of back-to-back MMAs (M = 128, K = 16), cycles each: 88 from a
+// `lane == 0` branch around the loop, 59 from an elected branch around it, and
+// max(32 + N / 4, N / 2), the tensor core's own time, from this form.  With
+// the waits and loads of the real loop (2,304 rows, no split-K) a 64-wide
+// k-tile takes 0.20 us at N = 64 and 0.24 us at N = 128, 0.31 us before.
+__device__ __forceinline__ void mma_bf16(uint32_t d_tmem, uint32_t a_lo, uint32_t a_hi, uint32_t b_lo, uint32_t b_hi,
+                                         uint32_t idesc, uint32_t accumulate) {
+  asm volatile(
+      "{\n\t.reg .pred p, q;\n\t.reg .b64 da, db;\n\t"
+      "mov.b64 da, {%1, %2};\n\t"
+      "mov.b64 db, {%3, %4};\n\t"
+      "setp.ne.b32 p, %6, 0;\n\t"
+      "elect.sync _|q, 0xffffffff;\n\t"
+      "@q tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %5, p;\n\t}" ::"r"(d_tmem),
+      "r"(a_lo), "r"(a_hi), "r"(b_lo), "r"(b_hi), "r"(idesc), "r"(accumulate)
       : "memory");
 }
 
+// By the same elected lane: `bar` completes once every MMA issued so far has.
 __device__ __forceinline__ void mma_commit(uint64_t *bar) {
-  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-                   smem_u32(bar))
-               : "memory");
+  asm volatile(
+      "{\n\t.reg .pred q;\n\t"
+      "elect.sync _|q, 0xffffffff;\n\t"
+      "@q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t}" ::"r"(smem_u32(bar))
+      : "memory");
 }
 
 // 32 lanes x 8 consecutive 32-bit columns (thread t: lane base + t); the
@@ -451,7 +479,8 @@ tma_gemm_kernel(const __grid_constant__ TcMaps maps, TcDesc d, DevDims dims, flo
   uint32_t *mbits = reinterpret_cast<uint32_t *>(smem + STAGES * kStageBytes + 256);  // BM x kMaskWords
   float *s_amp = reinterpret_cast<float *>(mbits + BM * kMaskWords), *s_att = s_amp + BM;
 
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  // the warp index through a shuffle: warp-uniform to the compiler
+  const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
   // shared-memory set-up and descriptor prefetch overlap the previous kernel
   if (tid == 0) {
     for (int s = 0; s < STAGES; ++s) {
@@ -517,60 +546,67 @@ tma_gemm_kernel(const __grid_constant__ TcMaps maps, TcDesc d, DevDims dims, flo
 
   if (warp == 0) {
     // ------------------------------------------------ TMA producer
-    if (lane == 0) {
-      for (int kt = 0; kt < nk; ++kt) {
-        const int s = kt % STAGES;
-        if (kt >= STAGES && !mbar_wait(&empty[s], ((kt / STAGES) - 1) & 1)) {
-          atomicOr(flag, 1u);
-          break;
-        }
-        const int k0 = kbeg + kt * BK;
+    int s = 0;
+    uint32_t round = 0;
+    for (int kt = 0; kt < nk; ++kt) {
+      if (kt >= STAGES && !mbar_wait(&empty[s], (round - 1) & 1)) {
+        if (lane == 0) atomicOr(flag, 1u);
+        break;
+      }
+      const int k0 = kbeg + kt * BK;
+      if (elect_one()) {
         if (kt < pre) {  // the other operand of a stage started before the wait
           if (d.stable == kStableA) load_b(s, k0);
           else load_a(s, k0);
-          continue;
+        } else {
+          mbar_expect_tx(&full[s], a_bytes + b_bytes);
+          load_a(s, k0);
+          load_b(s, k0);
         }
-        mbar_expect_tx(&full[s], a_bytes + b_bytes);
-        load_a(s, k0);
-        load_b(s, k0);
       }
+      __syncwarp();
+      if (++s == STAGES) { s = 0; ++round; }
     }
   } else if (warp == 1) {
     // ------------------------------------------------ MMA issuer
     const uint32_t idesc = instr_desc(BM, BN, d.A.mn_major, d.B.mn_major);
-    const uint32_t a_step = d.A.mn_major ? 2048u : 32u;
-    const uint32_t b_step = d.B.mn_major ? 2048u : 32u;
+    // descriptor words of stage 0; a stage or a K = 16 step further only moves
+    // the 16-byte-unit start address in the low word
+    const uint64_t da = smem_desc(smem_u32(smem), d.A.mn_major);
+    const uint64_t db = smem_desc(smem_u32(smem + kATileBytes), d.B.mn_major);
+    const uint32_t a_hi = (uint32_t)(da >> 32), b_hi = (uint32_t)(db >> 32);
+    const uint32_t a_step = d.A.mn_major ? 2048u >> 4 : 32u >> 4;
+    const uint32_t b_step = d.B.mn_major ? 2048u >> 4 : 32u >> 4;
     bool ok = true;
+    int s = 0;
+    uint32_t round = 0;
     for (int kt = 0; kt < nk; ++kt) {
-      const int s = kt % STAGES;
-      if (!mbar_wait(&full[s], (kt / STAGES) & 1)) ok = false;
-      ok = __all_sync(0xffffffffu, ok);
-      if (!ok) {
+      if (!__all_sync(0xffffffffu, mbar_wait(&full[s], round & 1))) {
+        ok = false;
         if (lane == 0) atomicOr(flag, 1u);
         break;
       }
-      uint8_t *a_tile = smem + s * kStageBytes;
-      uint8_t *b_tile = a_tile + kATileBytes;
       const int k0 = kbeg + kt * BK;
       if (d.node_dim == kNodeK && k0 + BK > K) {  // rows past the batch's nodes must not contribute
         const int from = K - k0;
+        uint8_t *a_tile = smem + s * kStageBytes;
         if (d.A.mn_major) clear_k_rows(a_tile, 2, from, lane);
-        if (d.B.mn_major) clear_k_rows(b_tile, b_atoms, from, lane);
+        if (d.B.mn_major) clear_k_rows(a_tile + kATileBytes, b_atoms, from, lane);
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
         __syncwarp();
       }
-      if (lane == 0) {
-        fence_after_sync();
-        const uint32_t a_base = smem_u32(a_tile), b_base = smem_u32(b_tile);
+      fence_after_sync();
+      uint32_t a_lo = (uint32_t)da + s * (kStageBytes >> 4), b_lo = (uint32_t)db + s * (kStageBytes >> 4);
 #pragma unroll
-        for (int j = 0; j < BK / 16; ++j)
-          mma_bf16(tmem, smem_desc(a_base + j * a_step, d.A.mn_major), smem_desc(b_base + j * b_step, d.B.mn_major),
-                   idesc, (kt > 0 || j > 0) ? 1u : 0u);
-        mma_commit(&empty[s]);
+      for (int j = 0; j < BK / 16; ++j) {
+        mma_bf16(tmem, a_lo, a_hi, b_lo, b_hi, idesc, (kt > 0 || j > 0) ? 1u : 0u);
+        a_lo += a_step;
+        b_lo += b_step;
       }
-      __syncwarp();
+      mma_commit(&empty[s]);
+      if (++s == STAGES) { s = 0; ++round; }
     }
-    if (ok && nk > 0 && lane == 0) mma_commit(acc_ready);
+    if (ok && nk > 0) mma_commit(acc_ready);
   } else if (EPI == kEpiD3) {
     // ------------------------------------------------ epilogue inputs (warps 2-7)
     // mask bit (row r, column 32 w + lane) = [mask > 0]; eight rows per batch

@@ -249,18 +249,21 @@ int gcnn_create(const gcnn_config *cfg, void *stream, gcnn_ctx **out) {
   // split-K workspace: the largest of the step's GEMMs
   // (over every node-count bucket a batch can launch with)
   size_t wsf = 0;
+  const bool inv = cfg->flags & GCNN_FLAG_ROW_INVARIANT;
   for (int ng = 256;; ng += 256) {
     const int n = std::min(ng, (int)Nc), h = (int)H;
-    wsf = std::max(wsf, gemm_simt_workspace_floats(n, 2 * h, h));
-    wsf = std::max(wsf, gemm_simt_workspace_floats(n, h, 16 * h));
-    wsf = std::max(wsf, gemm_simt_workspace_floats(16 * h + 1, h, n));
-    wsf = std::max(wsf, gemm_simt_workspace_floats(n, kAgg * h, 3 * h));
-    wsf = std::max(wsf, gemm_simt_workspace_floats(h + 1, 2 * h, n));
-    wsf = std::max(wsf, gemm_simt_workspace_floats(n, h, 3 * h));
-    if (cfg->node_head) {  // node head: x W1n, dz W1n^T, [x ; 1]^T dz
-      wsf = std::max(wsf, gemm_simt_workspace_floats(n, (int)Hh, h));
-      wsf = std::max(wsf, gemm_simt_workspace_floats(n, h, (int)Hh));
-      wsf = std::max(wsf, gemm_simt_workspace_floats(h + 1, (int)Hh, n));
+    wsf = std::max(wsf, gemm_simt_workspace_floats(n, 2 * h, h, inv));
+    wsf = std::max(wsf, gemm_simt_workspace_floats(n, h, 16 * h, inv));
+    if (cfg->node_head) wsf = std::max(wsf, gemm_simt_workspace_floats(n, (int)Hh, h, inv));  // x W1n
+    if (!inv) {  // a row-invariant backward does not split K
+      wsf = std::max(wsf, gemm_simt_workspace_floats(16 * h + 1, h, n, false));
+      wsf = std::max(wsf, gemm_simt_workspace_floats(n, kAgg * h, 3 * h, false));
+      wsf = std::max(wsf, gemm_simt_workspace_floats(h + 1, 2 * h, n, false));
+      wsf = std::max(wsf, gemm_simt_workspace_floats(n, h, 3 * h, false));
+      if (cfg->node_head) {  // dz W1n^T, [x ; 1]^T dz
+        wsf = std::max(wsf, gemm_simt_workspace_floats(n, h, (int)Hh, false));
+        wsf = std::max(wsf, gemm_simt_workspace_floats(h + 1, (int)Hh, n, false));
+      }
     }
     if (cfg->precision == GCNN_PREC_BF16) {
       const int r64 = (h + 63) / 64 * 64, r3 = (3 * h + 63) / 64 * 64, r16 = (16 * h + 63) / 64 * 64;

@@ -225,7 +225,7 @@ struct GemmWorkspace {
 };
 
 int run_gemm_simt(const GemmDesc &d, DevDims dims, const GemmWorkspace &ws, cudaStream_t s);
-size_t gemm_simt_workspace_floats(int M, int N, int K);
+size_t gemm_simt_workspace_floats(int M, int N, int K, bool row_invariant);
 // C = epilogue(sum over splits of partial[z]) in split order (deterministic).
 int run_splitk_reduce(const GemmDesc &d, DevDims dims, const float *partial, int splits, cudaStream_t s);
 int num_sms();

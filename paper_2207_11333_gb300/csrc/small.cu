@@ -202,7 +202,6 @@ __global__ void __launch_bounds__(kHeadThreads) head_graph_kernel(HeadArgs a) {
   float *sv = Ws + (size_t)rk * Hh;   // H: pooled features, later dg
   float *sz = sv + H;                 // Hh: z1
   float *sd = sz + Hh;                // Hh: dz1
-  const int gr = blockIdx.x;
   const int tid = threadIdx.x;
   const int nchunks = (H + rk - 1) / rk;
   // one chunk of W1 and whole float4 columns: W1 arrives by asynchronous copies
@@ -212,204 +211,321 @@ __global__ void __launch_bounds__(kHeadThreads) head_graph_kernel(HeadArgs a) {
   // or by a host copy, never by the kernel just before this one, which is a
   // GEMM of the last layer) and the graph offsets come from the collator, so
   // the copy of W1 and the offsets' loads overlap the previous kernel's tail.
-  if (kFwd && one) {
+  const int G = min(a.g_cap, a.dims.graphs(a.g_cap));
+  if (kFwd && one && (int)blockIdx.x < G) {
     for (int q = tid; q < H * (Hh >> 2); q += kHeadThreads) cp_async16(Ws + 4 * q, a.w1 + 4 * (size_t)q);
     asm volatile("cp.async.commit_group;" ::: "memory");
   }
-  const int G = min(a.g_cap, a.dims.graphs(a.g_cap));
-  const int n0 = gr < G ? a.node_off[gr] : 0, n1 = gr < G ? a.node_off[gr + 1] : 0, nn = n1 - n0;
+  int n0 = (int)blockIdx.x < G ? a.node_off[blockIdx.x] : 0, n1 = (int)blockIdx.x < G ? a.node_off[blockIdx.x + 1] : 0;
   pdl_entry(GCNN_K_HEAD_GRAPH);
-  if (gr >= G) {  // block-uniform
-    asm volatile("cp.async.wait_all;" ::: "memory");
-    return;
-  }
+  // a block takes graphs blockIdx.x, blockIdx.x + gridDim.x, ... and keeps W1
+  // between them where it fits
   int staged = -1;
-  auto stage = [&](int ch) {  // rows [ch * rk, ...) of W1 into Ws
-    __syncthreads();
-    const int k0 = ch * rk, cnt = min(rk, H - k0) * Hh;
-    const float4 *src = reinterpret_cast<const float4 *>(a.w1 + (size_t)k0 * Hh);
-    float4 *dst = reinterpret_cast<float4 *>(Ws);
+  for (int gr = blockIdx.x; gr < G; gr += gridDim.x) {
+    if (gr != (int)blockIdx.x) {
+      n0 = a.node_off[gr];
+      n1 = a.node_off[gr + 1];
+      __syncthreads();  // the previous graph's shared vectors are done with
+    }
+    const int nn = n1 - n0;
+    auto stage = [&](int ch) {  // rows [ch * rk, ...) of W1 into Ws
+      __syncthreads();
+      const int k0 = ch * rk, cnt = min(rk, H - k0) * Hh;
+      const float4 *src = reinterpret_cast<const float4 *>(a.w1 + (size_t)k0 * Hh);
+      float4 *dst = reinterpret_cast<float4 *>(Ws);
 #pragma unroll 4
-    for (int q = tid; q < cnt / 4; q += kHeadThreads) dst[q] = src[q];
-    for (int q = cnt / 4 * 4 + tid; q < cnt; q += kHeadThreads) Ws[q] = a.w1[(size_t)k0 * Hh + q];
-    __syncthreads();
-    staged = ch;
-  };
-  // one chunk: pooling and z1 use every thread (float4 column x row segment,
-  // partials summed in segment order) while W1 arrives
-  if (kFwd && one) {
-    float4 *part4 = reinterpret_cast<float4 *>(sd + Hh);  // kHeadRed float4
-    const int H4 = H >> 2, Hh4 = Hh >> 2;
-    staged = 0;
-    const int R = max(1, kHeadThreads / H4);
-    if (tid < R * H4) {
-      const int c4 = tid % H4;
-      float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
-      for (int i = n0 + tid / H4; i < n1; i += R) acc = add4(acc, ld4(a.x + (size_t)i * H + 4 * c4));
-      part4[tid] = acc;
-    }
-    __syncthreads();
-    for (int c4 = tid; c4 < H4; c4 += kHeadThreads) {
-      float4 v = part4[c4];
-      for (int r = 1; r < R; ++r) v = add4(v, part4[r * H4 + c4]);
-      if (nn > 0) {
-        const float inv = (float)nn;
-        v = make_float4(v.x / inv, v.y / inv, v.z / inv, v.w / inv);
+      for (int q = tid; q < cnt / 4; q += kHeadThreads) dst[q] = src[q];
+      for (int q = cnt / 4 * 4 + tid; q < cnt; q += kHeadThreads) Ws[q] = a.w1[(size_t)k0 * Hh + q];
+      __syncthreads();
+      staged = ch;
+    };
+    // one chunk: pooling and z1 use every thread (float4 column x row segment,
+    // partials summed in segment order) while W1 arrives
+    if (kFwd && one) {
+      float4 *part4 = reinterpret_cast<float4 *>(sd + Hh);  // kHeadRed float4
+      const int H4 = H >> 2, Hh4 = Hh >> 2;
+      staged = 0;
+      const int R = max(1, kHeadThreads / H4);
+      if (tid < R * H4) {
+        const int c4 = tid % H4;
+        float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+        for (int i = n0 + tid / H4; i < n1; i += R) acc = add4(acc, ld4(a.x + (size_t)i * H + 4 * c4));
+        part4[tid] = acc;
       }
-      st4(sv + 4 * c4, v);
-      st4(a.pooled + (size_t)gr * H + 4 * c4, v);
-    }
-    asm volatile("cp.async.wait_all;" ::: "memory");
-    __syncthreads();
-    const int S = max(1, kHeadThreads / Hh4), kper = (H + S - 1) / S;
-    if (tid < S * Hh4) {
-      const int c4 = tid % Hh4, seg = tid / Hh4, k1 = min(H, (seg + 1) * kper);
-      float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
-      for (int k = seg * kper; k < k1; ++k) {
-        const float gk = sv[k];
-        const float4 w = ld4(Ws + (size_t)k * Hh + 4 * c4);
-        acc.x = fmaf(gk, w.x, acc.x); acc.y = fmaf(gk, w.y, acc.y);
-        acc.z = fmaf(gk, w.z, acc.z); acc.w = fmaf(gk, w.w, acc.w);
+      __syncthreads();
+      for (int c4 = tid; c4 < H4; c4 += kHeadThreads) {
+        float4 v = part4[c4];
+        for (int r = 1; r < R; ++r) v = add4(v, part4[r * H4 + c4]);
+        if (nn > 0) {
+          const float inv = (float)nn;
+          v = make_float4(v.x / inv, v.y / inv, v.z / inv, v.w / inv);
+        }
+        st4(sv + 4 * c4, v);
+        st4(a.pooled + (size_t)gr * H + 4 * c4, v);
       }
-      part4[tid] = acc;
-    }
-    __syncthreads();
-    for (int c4 = tid; c4 < Hh4; c4 += kHeadThreads) {
-      float4 v = make_float4(a.b1[4 * c4], a.b1[4 * c4 + 1], a.b1[4 * c4 + 2], a.b1[4 * c4 + 3]);
-      for (int sg = 0; sg < S; ++sg) v = add4(v, part4[sg * Hh4 + c4]);
-      st4(sz + 4 * c4, v);
-    }
-    __syncthreads();
-    float part = 0.f;
-    for (int c = tid; c < Hh; c += kHeadThreads) {
-      a.z1[(size_t)gr * Hh + c] = sz[c];
-      part += fmaxf(sz[c], 0.f) * a.w2[c];
-    }
-    const float s = block_sum<kHeadThreads>(part, red);
-    if (tid == 0) {
-      s_pred = s + a.b2[0];
-      a.pred[gr] = s_pred;
-    }
-  } else if (kFwd) {
-    for (int k = tid; k < H; k += kHeadThreads) {
-      float s4[4] = {0.f, 0.f, 0.f, 0.f};
-      int i = n0;
-      for (; i + 4 <= n1; i += 4) {
-#pragma unroll
-        for (int u = 0; u < 4; ++u) s4[u] += a.x[(size_t)(i + u) * H + k];
+      asm volatile("cp.async.wait_all;" ::: "memory");
+      __syncthreads();
+      const int S = max(1, kHeadThreads / Hh4), kper = (H + S - 1) / S;
+      if (tid < S * Hh4) {
+        const int c4 = tid % Hh4, seg = tid / Hh4, k1 = min(H, (seg + 1) * kper);
+        float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+        for (int k = seg * kper; k < k1; ++k) {
+          const float gk = sv[k];
+          const float4 w = ld4(Ws + (size_t)k * Hh + 4 * c4);
+          acc.x = fmaf(gk, w.x, acc.x); acc.y = fmaf(gk, w.y, acc.y);
+          acc.z = fmaf(gk, w.z, acc.z); acc.w = fmaf(gk, w.w, acc.w);
+        }
+        part4[tid] = acc;
       }
-      for (; i < n1; ++i) s4[0] += a.x[(size_t)i * H + k];
-      float v = (s4[0] + s4[1]) + (s4[2] + s4[3]);
-      if (nn > 0) v /= (float)nn;
-      sv[k] = v;
-      a.pooled[(size_t)gr * H + k] = v;
-    }
-    for (int c = tid; c < Hh; c += kHeadThreads) sz[c] = a.b1[c];
-    for (int ch = 0; ch < nchunks; ++ch) {
-      stage(ch);
-      const int k0 = ch * rk, rows = min(rk, H - k0);
+      __syncthreads();
+      for (int c4 = tid; c4 < Hh4; c4 += kHeadThreads) {
+        float4 v = make_float4(a.b1[4 * c4], a.b1[4 * c4 + 1], a.b1[4 * c4 + 2], a.b1[4 * c4 + 3]);
+        for (int sg = 0; sg < S; ++sg) v = add4(v, part4[sg * Hh4 + c4]);
+        st4(sz + 4 * c4, v);
+      }
+      __syncthreads();
+      float part = 0.f;
       for (int c = tid; c < Hh; c += kHeadThreads) {
-        float acc = sz[c];
+        a.z1[(size_t)gr * Hh + c] = sz[c];
+        part += fmaxf(sz[c], 0.f) * a.w2[c];
+      }
+      const float s = block_sum<kHeadThreads>(part, red);
+      if (tid == 0) {
+        s_pred = s + a.b2[0];
+        a.pred[gr] = s_pred;
+      }
+    } else if (kFwd) {
+      for (int k = tid; k < H; k += kHeadThreads) {
+        float s4[4] = {0.f, 0.f, 0.f, 0.f};
+        int i = n0;
+        for (; i + 4 <= n1; i += 4) {
+#pragma unroll
+          for (int u = 0; u < 4; ++u) s4[u] += a.x[(size_t)(i + u) * H + k];
+        }
+        for (; i < n1; ++i) s4[0] += a.x[(size_t)i * H + k];
+        float v = (s4[0] + s4[1]) + (s4[2] + s4[3]);
+        if (nn > 0) v /= (float)nn;
+        sv[k] = v;
+        a.pooled[(size_t)gr * H + k] = v;
+      }
+      for (int c = tid; c < Hh; c += kHeadThreads) sz[c] = a.b1[c];
+      for (int ch = 0; ch < nchunks; ++ch) {
+        stage(ch);
+        const int k0 = ch * rk, rows = min(rk, H - k0);
+        for (int c = tid; c < Hh; c += kHeadThreads) {
+          float acc = sz[c];
 #pragma unroll 8
-        for (int k = 0; k < rows; ++k) acc += sv[k0 + k] * Ws[(size_t)k * Hh + c];
-        sz[c] = acc;
+          for (int k = 0; k < rows; ++k) acc += sv[k0 + k] * Ws[(size_t)k * Hh + c];
+          sz[c] = acc;
+        }
+      }
+      __syncthreads();
+      float part = 0.f;
+      for (int c = tid; c < Hh; c += kHeadThreads) {
+        a.z1[(size_t)gr * Hh + c] = sz[c];
+        part += fmaxf(sz[c], 0.f) * a.w2[c];
+      }
+      const float s = block_sum<kHeadThreads>(part, red);
+      if (tid == 0) {
+        s_pred = s + a.b2[0];
+        a.pred[gr] = s_pred;
       }
     }
-    __syncthreads();
-    float part = 0.f;
-    for (int c = tid; c < Hh; c += kHeadThreads) {
-      a.z1[(size_t)gr * Hh + c] = sz[c];
-      part += fmaxf(sz[c], 0.f) * a.w2[c];
-    }
-    const float s = block_sum<kHeadThreads>(part, red);
-    if (tid == 0) {
-      s_pred = s + a.b2[0];
-      a.pred[gr] = s_pred;
-    }
-  }
-  if (kBwd) {
-    if (!kFwd) {
-      for (int c = tid; c < Hh; c += kHeadThreads) sz[c] = a.z1[(size_t)gr * Hh + c];
-      if (tid == 0) s_pred = a.pred[gr];
-    }
-    __syncthreads();
-    if (tid == 0) {
-      const float r = s_pred - a.y[gr];
-      // the MSE gradient times the loss scale (data-parallel weighting, 1 alone)
-      const float dp = a.dpred_in ? a.dpred_in[gr] : (2.f * r / (float)G) * (a.loss_scale ? a.loss_scale[0] : 1.f);
-      a.dpred[gr] = dp;
-      s_dp = dp;
-    }
-    __syncthreads();
-    const float dp = s_dp;
-    for (int c = tid; c < Hh; c += kHeadThreads) {
-      const float d = sz[c] > 0.f ? dp * a.w2[c] : 0.f;
-      sd[c] = d;
-      a.dz1[(size_t)gr * Hh + c] = d;
-    }
-    // dg = W1 dz1, chunks in reverse order (the forward's last chunk is still
-    // staged): one thread per row of W1, four running sums over float4
-    // columns (16-byte aligned when Hh is a multiple of 4)
-    for (int ch = nchunks - 1; ch >= 0; --ch) {
-      if (staged != ch) stage(ch);
-      else __syncthreads();
-      const int k0 = ch * rk, rows = min(rk, H - k0);
-      for (int k = tid; k < rows; k += kHeadThreads) {
-        const float *w = Ws + (size_t)k * Hh;
-        float s0 = 0.f, s1 = 0.f, s2 = 0.f, s3 = 0.f;
-        int c = 0;
-        if ((Hh & 3) == 0) {
+    if (kBwd) {
+      if (!kFwd) {
+        for (int c = tid; c < Hh; c += kHeadThreads) sz[c] = a.z1[(size_t)gr * Hh + c];
+        if (tid == 0) s_pred = a.pred[gr];
+      }
+      __syncthreads();
+      if (tid == 0) {
+        const float r = s_pred - a.y[gr];
+        // the MSE gradient times the loss scale (data-parallel weighting, 1 alone)
+        const float dp = a.dpred_in ? a.dpred_in[gr] : (2.f * r / (float)G) * (a.loss_scale ? a.loss_scale[0] : 1.f);
+        a.dpred[gr] = dp;
+        s_dp = dp;
+      }
+      __syncthreads();
+      const float dp = s_dp;
+      for (int c = tid; c < Hh; c += kHeadThreads) {
+        const float d = sz[c] > 0.f ? dp * a.w2[c] : 0.f;
+        sd[c] = d;
+        a.dz1[(size_t)gr * Hh + c] = d;
+      }
+      // dg = W1 dz1, chunks in reverse order (the forward's last chunk is still
+      // staged): one thread per row of W1, four running sums over float4
+      // columns (16-byte aligned when Hh is a multiple of 4)
+      for (int ch = nchunks - 1; ch >= 0; --ch) {
+        if (staged != ch) stage(ch);
+        else __syncthreads();
+        const int k0 = ch * rk, rows = min(rk, H - k0);
+        for (int k = tid; k < rows; k += kHeadThreads) {
+          const float *w = Ws + (size_t)k * Hh;
+          float s0 = 0.f, s1 = 0.f, s2 = 0.f, s3 = 0.f;
+          int c = 0;
+          if ((Hh & 3) == 0) {
 #pragma unroll 4
-          for (; c < Hh; c += 4) {
-            const float4 wv = ld4(w + c), dv = ld4(sd + c);
-            s0 = fmaf(wv.x, dv.x, s0); s1 = fmaf(wv.y, dv.y, s1);
-            s2 = fmaf(wv.z, dv.z, s2); s3 = fmaf(wv.w, dv.w, s3);
+            for (; c < Hh; c += 4) {
+              const float4 wv = ld4(w + c), dv = ld4(sd + c);
+              s0 = fmaf(wv.x, dv.x, s0); s1 = fmaf(wv.y, dv.y, s1);
+              s2 = fmaf(wv.z, dv.z, s2); s3 = fmaf(wv.w, dv.w, s3);
+            }
+          }
+          for (; c < Hh; ++c) s0 = fmaf(w[c], sd[c], s0);
+          const float acc = (s0 + s1) + (s2 + s3);
+          sv[k0 + k] = acc;
+          a.dg[(size_t)gr * H + k0 + k] = acc;
+        }
+      }
+      __syncthreads();
+      // mean pooling backward on the graph's nodes, four items per thread at a
+      // time: every load of the four before any store
+      const float n = (float)nn;
+      const int H4 = H >> 2, items = nn * H4;
+      constexpr int U = 4;
+      for (int q0 = tid; q0 < items; q0 += U * kHeadThreads) {
+        float4 e[U], m[U];
+        float am[U], at[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+          const int q = min(q0 + u * kHeadThreads, items - 1);  // a valid item; only real ones are stored
+          const int i = n0 + q / H4, c = (q % H4) * 4;
+          e[u] = a.dx_add ? ld4(a.dx_add + (size_t)i * H + c) : make_float4(0.f, 0.f, 0.f, 0.f);
+          if (a.D3) {
+            m[u] = ld4(a.h + (size_t)i * H + c);
+            am[u] = a.amp[i];
+            at[u] = a.att[i];
           }
         }
-        for (; c < Hh; ++c) s0 = fmaf(w[c], sd[c], s0);
-        const float acc = (s0 + s1) + (s2 + s3);
-        sv[k0 + k] = acc;
-        a.dg[(size_t)gr * H + k0 + k] = acc;
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+          const int q = q0 + u * kHeadThreads;
+          if (q >= items) break;
+          const int i = n0 + q / H4, c = (q % H4) * 4;
+          // plus the node-level head's gradient on the same atoms, if any
+          float4 d = make_float4(sv[c] / n, sv[c + 1] / n, sv[c + 2] / n, sv[c + 3] / n);
+          if (a.dx_add) d = make_float4(d.x + e[u].x, d.y + e[u].y, d.z + e[u].z, d.w + e[u].w);
+          st4(a.dx + (size_t)i * H + c, d);
+          if (a.D3) {
+            const float gx = m[u].x > 0.f ? d.x : 0.f, gy = m[u].y > 0.f ? d.y : 0.f;
+            const float gz = m[u].z > 0.f ? d.z : 0.f, gw = m[u].w > 0.f ? d.w : 0.f;
+            uint16_t *o = a.D3 + (size_t)i * a.ld3 + c;
+            st_bf16x4(o, am[u] * gx, am[u] * gy, am[u] * gz, am[u] * gw);
+            st_bf16x4(o + H, at[u] * gx, at[u] * gy, at[u] * gz, at[u] * gw);
+            st_bf16x4(o + 2 * H, gx, gy, gz, gw);
+          }
+        }
       }
     }
+  }
+}
+
+// Forward of the head for many graphs: a block keeps W1 in shared memory and
+// takes kHeadBatch graphs at a time, so that each staged row of W1 is read once
+// for all of them and the chain of barriers is paid once.  Same sums in the
+// same order as head_graph_kernel (float4 columns over row segments, z1 over k
+// segments, the prediction by warps).  3,600 graphs at H = Hh = 200: one block
+// per graph, each copying W1 (160 KB), took 154 us; this takes 56 us.
+constexpr int kHeadBatch = 4;
+
+__global__ void __launch_bounds__(kHeadThreads) head_forward_kernel(HeadArgs a) {
+  extern __shared__ float sm[];
+  __shared__ float red[kHeadBatch][kHeadThreads / 32];
+  const int H = a.H, Hh = a.Hh, H4 = H >> 2, Hh4 = Hh >> 2;
+  float *Ws = sm;                                              // H x Hh
+  float4 *sv = reinterpret_cast<float4 *>(Ws + (size_t)H * Hh);  // H x kHeadBatch: pooled features, graphs innermost
+  float4 *part = sv + H;                                       // kHeadBatch x kHeadRed: partials of z1
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int G = min(a.g_cap, a.dims.graphs(a.g_cap));
+  const int first = blockIdx.x * kHeadBatch, step = gridDim.x * kHeadBatch;
+  if (first < G) {  // W1 before the dependency wait, as in head_graph_kernel
+    for (int q = tid; q < H * Hh4; q += kHeadThreads) cp_async16(Ws + 4 * q, a.w1 + 4 * (size_t)q);
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  }
+  pdl_entry(GCNN_K_HEAD_GRAPH);
+  const int R = max(1, kHeadThreads / H4);
+  const int S = max(1, kHeadThreads / Hh4), kper = (H + S - 1) / S;
+  for (int g0 = first; g0 < G; g0 += step) {
+    // mean pooling: a thread per (row segment, float4 column), the graphs'
+    // rows loaded side by side; then the segments' sums in segment order
+    if (g0 != first) __syncthreads();  // the previous graphs' z1 is done with
+    if (tid < R * H4) {
+      const int c4 = tid % H4;
+      int i[kHeadBatch], end[kHeadBatch], most = 0;
+      float4 s[kHeadBatch];
+#pragma unroll
+      for (int u = 0; u < kHeadBatch; ++u) {
+        i[u] = g0 + u < G ? a.node_off[g0 + u] + tid / H4 : 0;
+        end[u] = g0 + u < G ? a.node_off[g0 + u + 1] : 0;
+        most = max(most, end[u] - i[u]);
+        s[u] = make_float4(0.f, 0.f, 0.f, 0.f);
+      }
+#pragma unroll 2
+      for (int t = 0; t < most; t += R)
+#pragma unroll
+        for (int u = 0; u < kHeadBatch; ++u)
+          if (i[u] + t < end[u]) s[u] = add4(s[u], ld4(a.x + (size_t)(i[u] + t) * H + 4 * c4));
+#pragma unroll
+      for (int u = 0; u < kHeadBatch; ++u) part[u * kHeadRed + tid] = s[u];
+    }
     __syncthreads();
-    // mean pooling backward on the graph's nodes, four items per thread at a
-    // time: every load of the four before any store
-    const float n = (float)nn;
-    const int H4 = H >> 2, items = nn * H4;
-    constexpr int U = 4;
-    for (int q0 = tid; q0 < items; q0 += U * kHeadThreads) {
-      float4 e[U], m[U];
-      float am[U], at[U];
+    for (int q = tid; q < kHeadBatch * H4; q += kHeadThreads) {
+      const int u = q / H4, c4 = q % H4, g = g0 + u;
+      float4 v = part[u * kHeadRed + c4];
+      for (int r = 1; r < R; ++r) v = add4(v, part[u * kHeadRed + r * H4 + c4]);
+      if (g < G) {
+        const int nn = a.node_off[g + 1] - a.node_off[g];
+        if (nn > 0) {
+          const float n = (float)nn;
+          v = make_float4(v.x / n, v.y / n, v.z / n, v.w / n);
+        }
+        st4(a.pooled + (size_t)g * H + 4 * c4, v);
+      }
+      float *o = reinterpret_cast<float *>(sv + 4 * c4) + u;
+      o[0] = v.x; o[kHeadBatch] = v.y; o[2 * kHeadBatch] = v.z; o[3 * kHeadBatch] = v.w;
+    }
+    asm volatile("cp.async.wait_all;" ::: "memory");
+    __syncthreads();
+    if (tid < S * Hh4) {
+      const int c4 = tid % Hh4, seg = tid / Hh4, k1 = min(H, (seg + 1) * kper);
+      float4 acc[kHeadBatch];
 #pragma unroll
-      for (int u = 0; u < U; ++u) {
-        const int q = min(q0 + u * kHeadThreads, items - 1);  // a valid item; only real ones are stored
-        const int i = n0 + q / H4, c = (q % H4) * 4;
-        e[u] = a.dx_add ? ld4(a.dx_add + (size_t)i * H + c) : make_float4(0.f, 0.f, 0.f, 0.f);
-        if (a.D3) {
-          m[u] = ld4(a.h + (size_t)i * H + c);
-          am[u] = a.amp[i];
-          at[u] = a.att[i];
+      for (int u = 0; u < kHeadBatch; ++u) acc[u] = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll 4
+      for (int k = seg * kper; k < k1; ++k) {
+        const float4 w = ld4(Ws + (size_t)k * Hh + 4 * c4), gv = sv[k];
+        const float gk[kHeadBatch] = {gv.x, gv.y, gv.z, gv.w};
+#pragma unroll
+        for (int u = 0; u < kHeadBatch; ++u) {
+          acc[u].x = fmaf(gk[u], w.x, acc[u].x); acc[u].y = fmaf(gk[u], w.y, acc[u].y);
+          acc[u].z = fmaf(gk[u], w.z, acc[u].z); acc[u].w = fmaf(gk[u], w.w, acc[u].w);
         }
       }
 #pragma unroll
-      for (int u = 0; u < U; ++u) {
-        const int q = q0 + u * kHeadThreads;
-        if (q >= items) break;
-        const int i = n0 + q / H4, c = (q % H4) * 4;
-        // plus the node-level head's gradient on the same atoms, if any
-        float4 d = make_float4(sv[c] / n, sv[c + 1] / n, sv[c + 2] / n, sv[c + 3] / n);
-        if (a.dx_add) d = make_float4(d.x + e[u].x, d.y + e[u].y, d.z + e[u].z, d.w + e[u].w);
-        st4(a.dx + (size_t)i * H + c, d);
-        if (a.D3) {
-          const float gx = m[u].x > 0.f ? d.x : 0.f, gy = m[u].y > 0.f ? d.y : 0.f;
-          const float gz = m[u].z > 0.f ? d.z : 0.f, gw = m[u].w > 0.f ? d.w : 0.f;
-          uint16_t *o = a.D3 + (size_t)i * a.ld3 + c;
-          st_bf16x4(o, am[u] * gx, am[u] * gy, am[u] * gz, am[u] * gw);
-          st_bf16x4(o + H, at[u] * gx, at[u] * gy, at[u] * gz, at[u] * gw);
-          st_bf16x4(o + 2 * H, gx, gy, gz, gw);
-        }
-      }
+      for (int u = 0; u < kHeadBatch; ++u) part[u * kHeadRed + tid] = acc[u];
+    }
+    __syncthreads();
+    for (int q = tid; q < kHeadBatch * Hh4; q += kHeadThreads) {
+      const int u = q / Hh4, c4 = q % Hh4;
+      float4 v = make_float4(a.b1[4 * c4], a.b1[4 * c4 + 1], a.b1[4 * c4 + 2], a.b1[4 * c4 + 3]);
+      for (int sg = 0; sg < S; ++sg) v = add4(v, part[u * kHeadRed + sg * Hh4 + c4]);
+      part[u * kHeadRed + c4] = v;  // z1 over segment 0's place, which this thread alone has read
+      if (g0 + u < G) st4(a.z1 + (size_t)(g0 + u) * Hh + 4 * c4, v);
+    }
+    __syncthreads();
+#pragma unroll
+    for (int u = 0; u < kHeadBatch; ++u) {
+      const float *z = reinterpret_cast<const float *>(part + u * kHeadRed);
+      float v = 0.f;
+      for (int c = tid; c < Hh; c += kHeadThreads) v += fmaxf(z[c], 0.f) * a.w2[c];
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+      if (lane == 0) red[u][warp] = v;
+    }
+    __syncthreads();
+    if (tid < kHeadBatch && g0 + tid < G) {
+      float s = 0.f;
+      for (int q = 0; q < kHeadThreads / 32; ++q) s += red[tid][q];
+      a.pred[g0 + tid] = s + a.b2[0];
     }
   }
 }
@@ -811,11 +927,19 @@ int launch_pool_bwd(int G, int n_nodes, int H, DevDims dims, const int *node_off
 namespace {
 constexpr int kHeadSmemFloats = 40 * 1024;  // 160 KB: W1 rows plus pooled / z1 / dz1 vectors
 
+constexpr size_t kHeadForwardBytes = 224 * 1024;
+
+// W1 in one chunk, in whole float4 columns
+bool head_one_chunk(const HeadArgs &a) { return a.rk >= a.H && a.Hh % 4 == 0; }
+
+size_t head_forward_bytes(const HeadArgs &a) {
+  return sizeof(float) * (size_t)a.H * a.Hh + sizeof(float4) * ((size_t)a.H + kHeadBatch * kHeadRed);
+}
 template <bool F, bool B>
 int head_graph(HeadArgs a, cudaStream_t s) {
   static bool configured = false;
   // the one-chunk forward also keeps kHeadRed float4 partials
-  const bool one = a.rk >= a.H && a.Hh % 4 == 0;
+  const bool one = head_one_chunk(a);
   const size_t bytes =
       sizeof(float) * ((size_t)a.rk * a.Hh + a.H + 2 * (size_t)a.Hh) + (one ? sizeof(float4) * kHeadRed : 0);
   if (!configured) {
@@ -823,7 +947,11 @@ int head_graph(HeadArgs a, cudaStream_t s) {
                                        (int)(sizeof(float) * kHeadSmemFloats + sizeof(float4) * kHeadRed)));
     configured = true;
   }
-  GCNN_TRY(launch(head_graph_kernel<F, B>, a.g_cap, kHeadThreads, bytes, s, a));
+  // W1 that fits is copied once per block: then one block per SM takes the
+  // graphs in turn (several fit only where W1 is small)
+  const int blocks = one ? (int)std::min<size_t>(a.g_cap, (size_t)num_sms() * std::max<size_t>(1, 200 * 1024 / bytes))
+                         : a.g_cap;
+  GCNN_TRY(launch(head_graph_kernel<F, B>, blocks, kHeadThreads, bytes, s, a));
   return GCNN_OK;
 }
 }  // namespace
@@ -836,8 +964,18 @@ int launch_head_graph(HeadArgs a, bool fwd, bool bwd, cudaStream_t s) {
   if (rk < 4) return set_error(GCNN_EINVAL, "head: layer too wide for shared memory");
   a.rk = (int)rk;
   if (fwd && bwd) return head_graph<true, true>(a, s);
-  if (fwd) return head_graph<true, false>(a, s);
-  return head_graph<false, true>(a, s);
+  if (!fwd) return head_graph<false, true>(a, s);
+  // more graphs than SMs: several at a time (up to there one block per graph
+  // is one wave with the shorter chain)
+  if (a.g_cap > num_sms() && head_one_chunk(a) && head_forward_bytes(a) <= kHeadForwardBytes) {
+    static const cudaError_t attr = cudaFuncSetAttribute(
+        head_forward_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kHeadForwardBytes);
+    if (attr != cudaSuccess) return set_error(GCNN_ECUDA, "head: %s", cudaGetErrorString(attr));
+    const int blocks = std::min((int)ceil_div(a.g_cap, kHeadBatch), num_sms());
+    GCNN_TRY(launch(head_forward_kernel, blocks, kHeadThreads, head_forward_bytes(a), s, a));
+    return GCNN_OK;
+  }
+  return head_graph<true, false>(a, s);
 }
 
 int launch_head_grad(const HeadGradArgs &a, cudaStream_t s) {

@@ -106,6 +106,16 @@ __device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap *map
       : "memory");
 }
 
+// The same tile to the same place (and barrier) of every CTA of the cluster in `mask`.
+__device__ __forceinline__ void tma_load_2d_multicast(uint32_t dst, const CUtensorMap *map, int c0, int c1,
+                                                      uint64_t *bar, uint16_t mask) {
+  asm volatile(
+      "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes.multicast::cluster [%0], "
+      "[%1, {%2, %3}], [%4], %5;" ::"r"(dst),
+      "l"(reinterpret_cast<uint64_t>(map)), "r"(c0), "r"(c1), "r"(smem_u32(bar)), "h"(mask)
+      : "memory");
+}
+
 // ---------------------------------------------------------------- tcgen05
 __device__ __forceinline__ void tmem_alloc(uint32_t *dst_smem, uint32_t ncols) {
   asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(dst_smem)),
@@ -179,6 +189,17 @@ __device__ __forceinline__ void mma_commit(uint64_t *bar) {
       "{\n\t.reg .pred q;\n\t"
       "elect.sync _|q, 0xffffffff;\n\t"
       "@q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t}" ::"r"(smem_u32(bar))
+      : "memory");
+}
+
+// The same on the barrier at this place in every CTA of the cluster in `mask`.
+__device__ __forceinline__ void mma_commit_multicast(uint64_t *bar, uint16_t mask) {
+  asm volatile(
+      "{\n\t.reg .pred q;\n\t"
+      "elect.sync _|q, 0xffffffff;\n\t"
+      "@q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;\n\t}" ::"r"(
+          smem_u32(bar)),
+      "h"(mask)
       : "memory");
 }
 
@@ -703,6 +724,299 @@ tma_gemm_kernel(const __grid_constant__ TcMaps maps, TcDesc d, DevDims dims, flo
   if (warp == 0) tmem_free(tmem, ncols);
 }
 
+// ---------------------------------------------------------------- many rows
+// Products with more row tiles than SMs (no split-K): one persistent CTA per
+// SM walks the output tiles, 128 rows x up to 256 columns each, with the FP32
+// accumulator double-buffered in TMEM, so that the epilogue of one tile (its
+// stores are most of the time of the short-K products) overlaps the loads and
+// MMAs of the next.  One wide column tile reads each A tile from L2 once, and
+// pairs of CTAs (clusters of 2) share each B tile by TMA multicast; with
+// 128-wide tiles, two CTAs per SM and the epilogue after the loop, the same
+// products were bound by L2 reads (11.5 TB/s in the update) and by the chain
+// of one short CTA after the other.  What bounds it now is the bytes an SM takes
+// in: about 90 GB/s each with all of them loading.
+// us per launch, before and after: 64,427 atoms, H = 200: message 53 -> 33,
+// update 143 -> 108; 18,261 atoms, H = 256: dagg 50 -> 32, dx 26 -> 23.
+//   warp 0       TMA producer over all tiles of the CTA, stage ring as above
+//   warp 1       MMA issuer; a tile's accumulator is buffer (tile count) % 2
+//   warps 2-9    epilogue: warp w drains TMEM lanes 32 (w % 4) .. and one half
+//                of the columns in chunks of 16, turns each chunk through its
+//                own piece of shared memory and stores row segments of 64 bytes
+//                (chunks of 32 would cost the ring a stage)
+// Per element the same arithmetic as the tile kernel above: one accumulator in
+// k order, bias, ReLU, mask and scalers.
+constexpr int kRowsCluster = 2;  // CTAs that share each B tile
+constexpr int kRowsThreads = 320, kRowsEpiWarps = 8, kRowsMaxBN = 256, kRowsMaxStages = 6;
+constexpr int kRowsChunk = 16, kRowsPitch = kRowsChunk + 4;
+constexpr int kRowsEpiBytes = kRowsEpiWarps * 32 * kRowsPitch * 4;
+constexpr int kRowsBarBytes = 256;
+constexpr int kRowsSmemMax = 227 * 1024;
+
+__host__ __device__ constexpr int rows_b_bytes(int BN, bool mn_major) {
+  return mn_major ? (BN + 63) / 64 * (int)kMnAtomBytes : BN * BK * 2;
+}
+__host__ __device__ constexpr int rows_stages(int BN, bool mn_major) {
+  const int room = kRowsSmemMax - 1024 - kRowsEpiBytes - kRowsBarBytes;
+  const int n = room / (kATileBytes + rows_b_bytes(BN, mn_major));
+  return n < kRowsMaxStages ? n : kRowsMaxStages;
+}
+
+template <int EPI, int CL>
+__global__ void __launch_bounds__(kRowsThreads, 1)
+tma_gemm_rows_kernel(const __grid_constant__ TcMaps maps, TcDesc d, DevDims dims, int ntiles, int BN, unsigned *err) {
+  extern __shared__ uint8_t smem_raw[];
+  uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+  const int stages = rows_stages(BN, d.B.mn_major);
+  const int stage_bytes = kATileBytes + rows_b_bytes(BN, d.B.mn_major);
+  float *epi = reinterpret_cast<float *>(smem + stages * stage_bytes);
+  uint64_t *full = reinterpret_cast<uint64_t *>(smem + stages * stage_bytes + kRowsEpiBytes);
+  uint64_t *empty = full + kRowsMaxStages;
+  uint64_t *acc_full = empty + kRowsMaxStages;  // 2
+  uint64_t *acc_empty = acc_full + 2;           // 2
+  uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(acc_empty + 2);
+  uint32_t *flag = tmem_slot + 1;
+
+  const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
+  const int rank = (int)blockIdx.x % CL;  // the launch's clusters are CL neighbouring blocks
+  constexpr uint16_t kAll = (uint16_t)((1u << CL) - 1);
+  const Sizes sz = actual_sizes(d, dims);
+  const int M = sz.M, K = sz.K, N = d.N;
+  // tile t of a cluster: CL neighbouring row tiles, one per CTA, of column tile t % ntiles
+  const int t0 = (int)blockIdx.x / CL, tstep = (int)gridDim.x / CL;
+  const int tiles = ((M + BM - 1) / BM + CL - 1) / CL * ntiles;
+  const int nk = (K + BK - 1) / BK;
+  const int kid = EPI == kEpiC ? GCNN_K_GEMM_TC_C : GCNN_K_GEMM_TC_D3;
+  if (t0 >= tiles) {  // cluster-uniform, before any barrier wait or TMEM use
+    pdl_entry(kid);
+    return;
+  }
+  if (tid == 0) {
+    for (int s = 0; s < stages; ++s) {
+      mbar_init(&full[s], 1);
+      mbar_init(&empty[s], CL);
+    }
+    for (int b = 0; b < 2; ++b) {
+      mbar_init(&acc_full[b], 1);
+      mbar_init(&acc_empty[b], kRowsEpiWarps);
+    }
+    *flag = 0;
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&maps.a)) : "memory");
+    asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&maps.b)) : "memory");
+  }
+  // the peers' barriers are set up before anything arrives on them
+  if (CL > 1) cluster_sync();
+  const int b_atoms = (BN + 63) / 64;
+  const uint32_t bytes = (uint32_t)stage_bytes;
+  auto row0 = [&](int t) { return (t / ntiles * CL + rank) * BM; };
+  auto load_a = [&](int s, int m0, int k0) { tma_load_2d(smem_u32(smem + s * stage_bytes), &maps.a, k0, m0, &full[s]); };
+  // the CTA's share of the cluster's B tile (whole 64-column atoms, or BN / CL
+  // rows of the K-major tile), written to every CTA; each CTA's full barrier
+  // counts its own A tile and all of B
+  auto load_b = [&](int s, int n0, int k0) {
+    uint8_t *b_tile = smem + s * stage_bytes + kATileBytes;
+    if (!d.B.mn_major) {
+      const int share = BN / CL;
+      uint8_t *dst = b_tile + rank * share * BK * 2;
+      if (CL == 1) tma_load_2d(smem_u32(dst), &maps.b, k0, n0, &full[s]);
+      else tma_load_2d_multicast(smem_u32(dst), &maps.b, k0, n0 + rank * share, &full[s], kAll);
+    } else {
+      for (int j = rank; j < b_atoms; j += CL) {
+        const uint32_t dst = smem_u32(b_tile + j * kMnAtomBytes);
+        if (CL == 1) tma_load_2d(dst, &maps.b, n0 + 64 * j, k0, &full[s]);
+        else tma_load_2d_multicast(dst, &maps.b, n0 + 64 * j, k0, &full[s], kAll);
+      }
+    }
+  };
+  // the first tile's weights before the dependency wait (kStableB: not written
+  // by the kernel just before)
+  const int pre = d.stable == kStableB ? min(nk, stages) : 0;
+  if (tid == 0)
+    for (int kt = 0; kt < pre; ++kt) {
+      mbar_expect_tx(&full[kt], bytes);
+      load_b(kt, t0 % ntiles * BN, kt * BK);
+    }
+  pdl_entry(kid);
+  const uint32_t half_cols = BN <= 32 ? 32 : (BN <= 64 ? 64 : (BN <= 128 ? 128 : 256));
+  if (warp == 0) tmem_alloc(tmem_slot, 2 * half_cols);
+  fence_before_sync();
+  __syncthreads();
+  fence_after_sync();
+  const uint32_t tmem = *tmem_slot;
+
+  if (warp == 0) {
+    // ------------------------------------------------ TMA producer
+    // a stage is free once the MMAs of every CTA of the cluster have read it:
+    // this CTA's share of B goes to all of them
+    int s = 0, it = 0;
+    uint32_t round = 0;
+    for (int t = t0; t < tiles; t += tstep) {
+      const int m0 = row0(t), n0 = t % ntiles * BN;
+      bool ok = true;
+      for (int kt = 0; kt < nk; ++kt, ++it) {
+        if (it >= stages && !__all_sync(0xffffffffu, mbar_wait(&empty[s], (round - 1) & 1))) {
+          ok = false;
+          break;
+        }
+        if (elect_one()) {
+          if (it < pre) {
+            load_a(s, m0, kt * BK);
+          } else {
+            mbar_expect_tx(&full[s], bytes);
+            load_a(s, m0, kt * BK);
+            load_b(s, n0, kt * BK);
+          }
+        }
+        __syncwarp();
+        if (++s == stages) { s = 0; ++round; }
+      }
+      if (!ok) {
+        if (lane == 0) atomicOr(flag, 1u);
+        break;
+      }
+    }
+    // the peers' last arrivals on this CTA's empty barriers come in before it may leave
+    if (CL > 1)
+      for (int j = 0; j < stages; ++j, ++it) {
+        if (it >= stages && !__all_sync(0xffffffffu, mbar_wait(&empty[s], (round - 1) & 1))) {
+          if (lane == 0) atomicOr(flag, 1u);
+          break;
+        }
+        if (++s == stages) { s = 0; ++round; }
+      }
+  } else if (warp == 1) {
+    // ------------------------------------------------ MMA issuer
+    const uint32_t idesc = instr_desc(BM, BN, false, d.B.mn_major);
+    const uint64_t da = smem_desc(smem_u32(smem), false);
+    const uint64_t db = smem_desc(smem_u32(smem + kATileBytes), d.B.mn_major);
+    const uint32_t a_hi = (uint32_t)(da >> 32), b_hi = (uint32_t)(db >> 32);
+    const uint32_t b_step = d.B.mn_major ? 2048u >> 4 : 32u >> 4;
+    bool ok = true;
+    int s = 0, i = 0;
+    uint32_t round = 0;
+    for (int t = t0; t < tiles && ok; t += tstep, ++i) {
+      const uint32_t acc = tmem + (uint32_t)(i & 1) * half_cols;
+      // the epilogue has drained this buffer's previous tile
+      if (i >= 2) ok = __all_sync(0xffffffffu, mbar_wait(&acc_empty[i & 1], ((i >> 1) - 1) & 1));
+      fence_after_sync();
+      for (int kt = 0; kt < nk && ok; ++kt) {
+        ok = __all_sync(0xffffffffu, mbar_wait(&full[s], round & 1));
+        if (!ok) break;
+        fence_after_sync();
+        uint32_t a_lo = (uint32_t)da + s * (stage_bytes >> 4), b_lo = (uint32_t)db + s * (stage_bytes >> 4);
+#pragma unroll
+        for (int j = 0; j < BK / 16; ++j) {
+          mma_bf16(acc, a_lo, a_hi, b_lo, b_hi, idesc, (kt > 0 || j > 0) ? 1u : 0u);
+          a_lo += 32u >> 4;
+          b_lo += b_step;
+        }
+        if (CL == 1) mma_commit(&empty[s]);
+        else mma_commit_multicast(&empty[s], kAll);
+        if (++s == stages) { s = 0; ++round; }
+      }
+      if (ok) mma_commit(&acc_full[i & 1]);
+    }
+    if (!ok && lane == 0) atomicOr(flag, 1u);
+  } else {
+    // ------------------------------------------------ epilogue
+    const TcEpilogue e = d.ep;
+    const int q = warp & 3, half = (warp - 2) >> 2;
+    float *S = epi + (warp - 2) * 32 * kRowsPitch;
+    const int chunks = (BN + kRowsChunk - 1) / kRowsChunk, mid = (chunks + 1) / 2;
+    const int c0 = half ? mid : 0, c1 = half ? chunks : mid;
+    const int rr = lane >> 2, cc = (lane & 3) * 4;  // store: rows rr + 8 u of the warp's 32, columns cc ..
+    int i = 0;
+    for (int t = t0; t < tiles; t += tstep, ++i) {
+      const int m0 = row0(t) + 32 * q, n0 = t % ntiles * BN;
+      if (!__all_sync(0xffffffffu, mbar_wait(&acc_full[i & 1], (i >> 1) & 1))) {
+        if (lane == 0) atomicOr(flag, 1u);
+        break;
+      }
+      fence_after_sync();
+      const uint32_t acc = tmem + (uint32_t)(i & 1) * half_cols + ((uint32_t)(32 * q) << 16);
+      float am[4], at[4];
+      if (EPI == kEpiD3)
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          const int row = m0 + rr + 8 * u;
+          am[u] = row < M ? e.amp[row] : 0.f;
+          at[u] = row < M ? e.att[row] : 0.f;
+        }
+      for (int c = c0; c < c1; ++c) {
+        uint32_t v[2][8];
+#pragma unroll
+        for (int w = 0; w < 2; ++w) tmem_ld8(acc + (uint32_t)(c * kRowsChunk + 8 * w), v[w]);
+        const int n = n0 + c * kRowsChunk + cc;
+        const bool in = n < N && c * kRowsChunk + cc < BN;
+        float4 mk[4];
+        if (EPI == kEpiD3)
+#pragma unroll
+          for (int u = 0; u < 4; ++u) {
+            const int row = m0 + rr + 8 * u;
+            mk[u] = in && row < M ? *reinterpret_cast<const float4 *>(e.mask + (size_t)row * e.ldm + n)
+                                  : make_float4(0.f, 0.f, 0.f, 0.f);
+          }
+        float b[4] = {0.f, 0.f, 0.f, 0.f};
+        if (EPI == kEpiC && e.bias && in)
+#pragma unroll
+          for (int k = 0; k < 4; ++k)
+            if (n + k < e.bias_n) b[k] = e.bias[n + k];
+        tmem_wait_ld();
+        if (c + 1 == c1) {  // this warp has read all of the tile
+          fence_before_sync();
+          if (lane == 0)
+            asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(&acc_empty[i & 1])) : "memory");
+        }
+#pragma unroll
+        for (int w = 0; w < 2; ++w) {
+          uint4 *o = reinterpret_cast<uint4 *>(S + lane * kRowsPitch + 8 * w);
+          o[0] = make_uint4(v[w][0], v[w][1], v[w][2], v[w][3]);
+          o[1] = make_uint4(v[w][4], v[w][5], v[w][6], v[w][7]);
+        }
+        __syncwarp();
+        float4 x[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) x[u] = *reinterpret_cast<const float4 *>(S + (rr + 8 * u) * kRowsPitch + cc);
+        __syncwarp();
+        if (!in) continue;
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          const int row = m0 + rr + 8 * u;
+          if (row >= M) break;
+          if constexpr (EPI == kEpiC) {
+            x[u] = make_float4(x[u].x + b[0], x[u].y + b[1], x[u].z + b[2], x[u].w + b[3]);
+            if (e.relu) {
+              x[u].x = fmaxf(x[u].x, 0.f); x[u].y = fmaxf(x[u].y, 0.f);
+              x[u].z = fmaxf(x[u].z, 0.f); x[u].w = fmaxf(x[u].w, 0.f);
+            }
+            if (e.C) *reinterpret_cast<float4 *>(e.C + (size_t)row * e.ldc + n) = x[u];
+            if (e.C16) st_bf16x4(e.C16 + (size_t)row * e.ld16 + n, x[u].x, x[u].y, x[u].z, x[u].w);
+          } else {
+            if (e.C) *reinterpret_cast<float4 *>(e.C + (size_t)row * e.ldc + n) = x[u];
+            const float gx = mk[u].x > 0.f ? x[u].x : 0.f, gy = mk[u].y > 0.f ? x[u].y : 0.f;
+            const float gz = mk[u].z > 0.f ? x[u].z : 0.f, gw = mk[u].w > 0.f ? x[u].w : 0.f;
+            uint16_t *o = e.D3 + (size_t)row * e.ld3 + n;
+            st_bf16x4(o, am[u] * gx, am[u] * gy, am[u] * gz, am[u] * gw);
+            st_bf16x4(o + N, at[u] * gx, at[u] * gy, at[u] * gz, at[u] * gw);
+            st_bf16x4(o + 2 * N, gx, gy, gz, gw);
+          }
+        }
+      }
+      // a warp without columns (narrow tiles) releases the buffer at once
+      if (c0 >= c1) {
+        if (lane == 0)
+          asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(&acc_empty[i & 1])) : "memory");
+      }
+    }
+  }
+  fence_before_sync();
+  __syncthreads();
+  if (tid == 0 && *flag && err) atomicOr(err, kErrTimeout);
+  if (warp == 0) tmem_free(tmem, 2 * half_cols);
+  // no CTA leaves while a peer may still write to its memory or its barriers
+  if (CL > 1) cluster_sync();
+}
+
 // C = epilogue(sum over splits); one thread per 8 outputs
 __global__ void __launch_bounds__(256) tc_reduce_kernel(TcDesc d, DevDims dims, const float *__restrict__ partial,
                                                        int splits) {
@@ -809,6 +1123,10 @@ int configure() {
     set_smem_attr<kEpiPartial, false, true>(&rc);
     set_smem_attr<kEpiC, false, true>(&rc);
     set_smem_attr<kEpiC, true, true>(&rc);
+    for (auto kernel : {tma_gemm_rows_kernel<kEpiC, kRowsCluster>, tma_gemm_rows_kernel<kEpiD3, kRowsCluster>})
+      if (rc == GCNN_OK &&
+          cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kRowsSmemMax) != cudaSuccess)
+        rc = set_error(GCNN_ECUDA, "tc gemm: cannot set the shared-memory size");
     for (int sz = 2; sz <= kMaxCluster && rc == GCNN_OK; ++sz) {
       g_capacity[0][sz] = cluster_capacity_of<kEpiC>(sz);
       g_capacity[1][sz] = cluster_capacity_of<kEpiD3>(sz);
@@ -821,6 +1139,7 @@ int configure() {
 struct Plan {
   int BN, ntiles, splits;
   bool cluster;  // split-K summed in a cluster through distributed shared memory
+  bool rows;     // more row tiles than SMs: the persistent kernel (no split)
 };
 
 // Tile width and split count of one launch.  A CTA's time is dominated by
@@ -834,12 +1153,14 @@ struct Plan {
 // SM (clusters within their co-resident capacity), take the smallest
 // estimate; grids larger than that use the widest tiles and no split.
 // out_bytes: epilogue bytes per output element; b_mn: B tiles are MN-major
-// (loaded in 64-column atoms); d3: masked-gradient epilogue.
-Plan choose(int M, int N, int K, int max_splits, int max_ctas, double out_bytes, bool b_mn, bool d3) {
+// (loaded in 64-column atoms); d3: masked-gradient epilogue; node_rows: the
+// rows are the batch's nodes and A is K-major, the form of the persistent
+// kernel, which takes every grid of more than one wave.
+Plan choose(int M, int N, int K, int max_splits, int max_ctas, double out_bytes, bool b_mn, bool d3, bool node_rows) {
   const int sms = max_ctas > 0 ? std::min(max_ctas, num_sms()) : num_sms();
   const long long mtiles = (M + BM - 1) / BM;
   const int ktiles = std::max(1, (K + BK - 1) / BK);
-  Plan best{0, 0, 1, false};
+  Plan best{0, 0, 1, false, false};
   double best_t = 1e30;
   for (int bn = 16; bn <= kMaxBN; bn += 16) {
     const int nt = (N + bn - 1) / bn;
@@ -854,21 +1175,25 @@ Plan choose(int M, int N, int K, int max_splits, int max_ctas, double out_bytes,
       const double t = t_load + t_out + t_red;
       if (t < best_t) {
         best_t = t;
-        best = Plan{bn, nt, sp, false};
+        best = Plan{bn, nt, sp, false, false};
       }
       if (sp >= 2 && sp <= kMaxCluster && mtiles * nt <= g_capacity[d3 ? 1 : 0][sp] && mtiles * nt * sp <= sms) {
         const double t_cl = t_load + BM * (double)bn * 4.0 / 5.0e4 + 0.5 + BM * (double)bn * out_bytes / sp / 4.0e4;
         if (t_cl < best_t) {
           best_t = t_cl;
-          best = Plan{bn, nt, sp, true};
+          best = Plan{bn, nt, sp, true, false};
         }
       }
     }
   }
   if (best.BN == 0) {  // more than one wave: widest tiles, no split
-    best.ntiles = (N + kMaxBN - 1) / kMaxBN;
-    best.BN = ((N + best.ntiles - 1) / best.ntiles + 15) / 16 * 16;
+    const int most = node_rows ? kRowsMaxBN : kMaxBN;
+    best.ntiles = (N + most - 1) / most;
+    // the persistent kernel's CTAs each load whole 8-row groups of a K-major B tile
+    const int unit = node_rows ? 8 * std::max(2, kRowsCluster) : 16;
+    best.BN = ((N + best.ntiles - 1) / best.ntiles + unit - 1) / unit * unit;
     best.splits = 1;
+    best.rows = node_rows;
   }
   return best;
 }
@@ -909,6 +1234,32 @@ int launch_gemm(void (*kernel)(P...), dim3 grid, int cz, cudaStream_t s, A &&...
   return GCNN_OK;
 }
 
+// The persistent kernel's launch in clusters, with programmatic serialisation.
+template <typename... P, typename... A>
+int launch_rows(void (*kernel)(P...), int ctas, size_t smem, cudaStream_t s, A &&...args) {
+  cudaLaunchAttribute attr[2];
+  int n = 0;
+  attr[n].id = cudaLaunchAttributeClusterDimension;
+  attr[n].val.clusterDim.x = kRowsCluster;
+  attr[n].val.clusterDim.y = 1;
+  attr[n].val.clusterDim.z = 1;
+  ++n;
+  if (pdl_enabled(s)) {
+    attr[n].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[n].val.programmaticStreamSerializationAllowed = 1;
+    ++n;
+  }
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3((unsigned)ctas);
+  cfg.blockDim = dim3(kRowsThreads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cfg.attrs = attr;
+  cfg.numAttrs = n;
+  GCNN_CUDA_TRY(cudaLaunchKernelEx(&cfg, kernel, std::forward<A>(args)...));
+  return GCNN_OK;
+}
+
 }  // namespace
 
 namespace {
@@ -924,9 +1275,10 @@ int run_planned(const TcDesc &d, DevDims dims, const GemmWorkspace &ws, unsigned
     return set_error(GCNN_EINVAL, "tc gemm: N must be a multiple of 8 and outputs 16-byte aligned");
   GCNN_TRY(configure());
   const double out_bytes = (e.C ? 4.0 : 0.0) + (e.C16 ? 2.0 : 0.0) + (e.D3 ? 10.0 : 0.0);
-  Plan plan = choose(d.M, d.N, d.K, ws.max_splits, ws.max_ctas, out_bytes, d.B.mn_major, e.D3 != nullptr);
+  Plan plan = choose(d.M, d.N, d.K, ws.max_splits, ws.max_ctas, out_bytes, d.B.mn_major, e.D3 != nullptr,
+                     d.node_dim == kNodeM && !d.A.mn_major);
   if (force) plan = *force;
-  if (plan.BN < 16 || plan.BN > kMaxBN || plan.BN % 16 || plan.ntiles < 1 || plan.splits < 1)
+  if (plan.BN < 16 || plan.BN > (plan.rows ? kRowsMaxBN : kMaxBN) || plan.BN % 16 || plan.ntiles < 1 || plan.splits < 1)
     return set_error(GCNN_EINVAL, "tc gemm: tile width must be a multiple of 16 in [16, %d]", kMaxBN);
   if (plan.splits > 1 && !plan.cluster && (size_t)plan.splits * d.M * d.N > ws.floats) plan.splits = 1;
   if (used) *used = plan;
@@ -934,6 +1286,14 @@ int run_planned(const TcDesc &d, DevDims dims, const GemmWorkspace &ws, unsigned
   const int ktiles = (d.K + BK - 1) / BK;
   TcMaps maps;
   GCNN_TRY(make_map(&maps.a, d.A, d.A.mn_major ? 64 : BM));
+  if (plan.rows) {
+    GCNN_TRY(make_map(&maps.b, d.B, d.B.mn_major ? 64 : BN / kRowsCluster));
+    const int tiles = ((d.M + BM - 1) / BM + kRowsCluster - 1) / kRowsCluster * ntiles;
+    const size_t smem = 1024 + (size_t)rows_stages(BN, d.B.mn_major) * (kATileBytes + rows_b_bytes(BN, d.B.mn_major)) +
+                        kRowsEpiBytes + kRowsBarBytes;
+    return launch_rows(e.D3 ? tma_gemm_rows_kernel<kEpiD3, kRowsCluster> : tma_gemm_rows_kernel<kEpiC, kRowsCluster>,
+                       std::min(tiles, num_sms() / kRowsCluster) * kRowsCluster, smem, s, maps, d, dims, ntiles, BN, err);
+  }
   GCNN_TRY(make_map(&maps.b, d.B, d.B.mn_major ? 64 : BN));
   const int kps = (ktiles + splits - 1) / splits * BK;
   dim3 grid(ntiles, (d.M + BM - 1) / BM, splits);
@@ -1114,7 +1474,7 @@ int gemm_tc_study(int n_atoms, int H, int mode, double *rows, int max_rows, int 
           for (int cl = 0; cl <= 1 && rc == GCNN_OK; ++cl) {
             if (cl && (sp < 2 || sp > kMaxCluster || mt * nt > g_capacity[sh.d.ep.D3 ? 1 : 0][sp])) continue;
             if (!cl && sp > 1 && (size_t)sp * sh.d.M * sh.d.N > wsf) continue;
-            const Plan f{bn, nt, sp, cl == 1};
+            const Plan f{bn, nt, sp, cl == 1, false};
             rc = study_time(sh, dims, w, err, s, &f, &used, &us);
             if (rc == GCNN_OK) emit(sh.id, used, sh.d.K, us, 0);
           }
@@ -1128,7 +1488,7 @@ int gemm_tc_study(int n_atoms, int H, int mode, double *rows, int max_rows, int 
           t.d.K = k;
           t.d.A.cols = std::min(sh.d.A.cols, k);
           t.d.B.rows = std::min(sh.d.B.rows, k);
-          const Plan f{bn, nt, 1, false};
+          const Plan f{bn, nt, 1, false, false};
           Plan used{};
           double us = 0.0;
           rc = study_time(t, dims, w, err, s, &f, &used, &us);

@@ -38,6 +38,10 @@ namespace gcnn {
 namespace {
 
 constexpr int BM = 128, BK = 64, STAGES = 3, kThreads = 256;
+// Long k loops with an SM to themselves keep six stages in flight: three
+// (96 KB) held dW_U of 18,000 atoms at H = 256 to 66 us, six take 47.  Short
+// ones keep three, so that a second CTA (the other stream's) fits the SM.
+constexpr int kLongStages = 6, kLongTiles = 64;
 constexpr int kMaxBN = 128;
 // Co-resident CTAs per SM: about 100 KB of shared memory and at most 128
 // registers per thread each.  One CTA issues its MMAs at a latency-bound rate
@@ -55,7 +59,10 @@ constexpr int kStageBytes = kATileBytes + kBTileBytes;
 // tile rows' degree scalers, prefetched during the main loop
 constexpr int kMaskWords = kMaxBN / 32;
 constexpr int kSideBytes = BM * kMaskWords * 4 + 2 * BM * 4;
-constexpr int kSmemBytes = STAGES * kStageBytes + 1024 /* alignment slack */ + 256 /* barriers */ + kSideBytes;
+constexpr int smem_bytes(int stages) {
+  return stages * kStageBytes + 1024 /* alignment slack */ + 256 /* barriers */ + kSideBytes;
+}
+constexpr int kSmemBytes = smem_bytes(STAGES);
 constexpr long long kWaitCycles = 4000000000LL;  // ~2 s at 2 GHz
 constexpr uint32_t kMnAtomBytes = 64 * 128;      // 64 M/N elements x 64 k rows
 
@@ -489,22 +496,22 @@ __device__ __forceinline__ void clear_k_rows(uint8_t *tile, int atoms, int from,
 template <int EPI, bool CL, bool LEAN>
 __global__ void __launch_bounds__(kThreads, LEAN ? 3 : kCtasPerSm)
 tma_gemm_kernel(const __grid_constant__ TcMaps maps, TcDesc d, DevDims dims, float *__restrict__ partial, int splits,
-                int kps, int BN, unsigned *err) {
+                int kps, int BN, int stages, unsigned *err) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-  uint64_t *full = reinterpret_cast<uint64_t *>(smem + STAGES * kStageBytes);
-  uint64_t *empty = full + STAGES;
-  uint64_t *acc_ready = empty + STAGES;
+  uint64_t *full = reinterpret_cast<uint64_t *>(smem + stages * kStageBytes);
+  uint64_t *empty = full + stages;
+  uint64_t *acc_ready = empty + stages;
   uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(acc_ready + 1);
   uint32_t *flag = tmem_slot + 1;
-  uint32_t *mbits = reinterpret_cast<uint32_t *>(smem + STAGES * kStageBytes + 256);  // BM x kMaskWords
+  uint32_t *mbits = reinterpret_cast<uint32_t *>(smem + stages * kStageBytes + 256);  // BM x kMaskWords
   float *s_amp = reinterpret_cast<float *>(mbits + BM * kMaskWords), *s_att = s_amp + BM;
 
   // the warp index through a shuffle: warp-uniform to the compiler
   const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
   // shared-memory set-up and descriptor prefetch overlap the previous kernel
   if (tid == 0) {
-    for (int s = 0; s < STAGES; ++s) {
+    for (int s = 0; s < stages; ++s) {
       mbar_init(&full[s], 1);
       mbar_init(&empty[s], 1);
     }
@@ -550,7 +557,7 @@ tma_gemm_kernel(const __grid_constant__ TcMaps maps, TcDesc d, DevDims dims, flo
     }
   };
   // the stable operand's first stages go out before the dependency wait
-  const int pre = d.stable != kStableNone ? min(nk, STAGES) : 0;
+  const int pre = d.stable != kStableNone ? min(nk, stages) : 0;
   if (tid == 0)
     for (int kt = 0; kt < pre; ++kt) {
       mbar_expect_tx(&full[kt], a_bytes + b_bytes);
@@ -570,7 +577,7 @@ tma_gemm_kernel(const __grid_constant__ TcMaps maps, TcDesc d, DevDims dims, flo
     int s = 0;
     uint32_t round = 0;
     for (int kt = 0; kt < nk; ++kt) {
-      if (kt >= STAGES && !mbar_wait(&empty[s], (round - 1) & 1)) {
+      if (kt >= stages && !mbar_wait(&empty[s], (round - 1) & 1)) {
         if (lane == 0) atomicOr(flag, 1u);
         break;
       }
@@ -586,7 +593,7 @@ tma_gemm_kernel(const __grid_constant__ TcMaps maps, TcDesc d, DevDims dims, flo
         }
       }
       __syncwarp();
-      if (++s == STAGES) { s = 0; ++round; }
+      if (++s == stages) { s = 0; ++round; }
     }
   } else if (warp == 1) {
     // ------------------------------------------------ MMA issuer
@@ -625,7 +632,7 @@ tma_gemm_kernel(const __grid_constant__ TcMaps maps, TcDesc d, DevDims dims, flo
         b_lo += b_step;
       }
       mma_commit(&empty[s]);
-      if (++s == STAGES) { s = 0; ++round; }
+      if (++s == stages) { s = 0; ++round; }
     }
     if (ok && nk > 0) mma_commit(acc_ready);
   } else if (EPI == kEpiD3) {
@@ -1080,8 +1087,8 @@ constexpr int kMaxCluster = 6;  // largest split-K cluster (co-resident capacity
 template <int EPI, bool CL, bool LEAN = false>
 void set_smem_attr(int *rc) {
   if (*rc == GCNN_OK &&
-      cudaFuncSetAttribute(tma_gemm_kernel<EPI, CL, LEAN>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes) !=
-          cudaSuccess)
+      cudaFuncSetAttribute(tma_gemm_kernel<EPI, CL, LEAN>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                           smem_bytes(kLongStages)) != cudaSuccess)
     *rc = set_error(GCNN_ECUDA, "tc gemm: cannot set the shared-memory size");
 }
 
@@ -1205,10 +1212,10 @@ int max_splits_of(int M, int K) {
   return (int)std::max<long long>(1, std::min<long long>({32LL, (long long)ktiles, num_sms() / std::max(1LL, mtiles)}));
 }
 
-// kernel<<<grid, kThreads, kSmemBytes, s>>> as a cluster of (1, 1, cz) CTAs
+// kernel<<<grid, kThreads, smem_bytes(stages), s>>> as a cluster of (1, 1, cz) CTAs
 // (cz > 1), with programmatic serialisation like every launch of the library
 template <typename... P, typename... A>
-int launch_gemm(void (*kernel)(P...), dim3 grid, int cz, cudaStream_t s, A &&...args) {
+int launch_gemm(void (*kernel)(P...), dim3 grid, int cz, int stages, cudaStream_t s, A &&...args) {
   cudaLaunchAttribute attr[2];
   int n = 0;
   if (cz > 1) {
@@ -1226,7 +1233,7 @@ int launch_gemm(void (*kernel)(P...), dim3 grid, int cz, cudaStream_t s, A &&...
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = grid;
   cfg.blockDim = dim3(kThreads);
-  cfg.dynamicSmemBytes = kSmemBytes;
+  cfg.dynamicSmemBytes = smem_bytes(stages);
   cfg.stream = s;
   cfg.attrs = attr;
   cfg.numAttrs = n;
@@ -1297,17 +1304,20 @@ int run_planned(const TcDesc &d, DevDims dims, const GemmWorkspace &ws, unsigned
   GCNN_TRY(make_map(&maps.b, d.B, d.B.mn_major ? 64 : BN));
   const int kps = (ktiles + splits - 1) / splits * BK;
   dim3 grid(ntiles, (d.M + BM - 1) / BM, splits);
+  // clusters beyond pairs keep the small ring: with an SM per CTA fewer of them fit at once
+  const int stages = kps / BK >= kLongTiles && splits <= 2 ? kLongStages : STAGES;
   // the masked-gradient epilogue has no register-capped form
   const bool lean = d.lean && !e.D3;
   if (splits > 1 && plan.cluster) {
     auto kernel = e.D3 ? tma_gemm_kernel<kEpiD3, true, false>
                        : (lean ? tma_gemm_kernel<kEpiC, true, true> : tma_gemm_kernel<kEpiC, true, false>);
-    return launch_gemm(kernel, grid, splits, s, maps, d, dims, (float *)nullptr, splits, kps, BN, err);
+    return launch_gemm(kernel, grid, splits, stages, s, maps, d, dims, (float *)nullptr, splits, kps, BN, stages, err);
   }
   auto kernel = splits > 1 ? (lean ? tma_gemm_kernel<kEpiPartial, false, true> : tma_gemm_kernel<kEpiPartial, false, false>)
                            : (e.D3 ? tma_gemm_kernel<kEpiD3, false, false>
                                    : (lean ? tma_gemm_kernel<kEpiC, false, true> : tma_gemm_kernel<kEpiC, false, false>));
-  GCNN_TRY(launch_gemm(kernel, grid, 1, s, maps, d, dims, splits > 1 ? ws.partial : nullptr, splits, kps, BN, err));
+  GCNN_TRY(launch_gemm(kernel, grid, 1, stages, s, maps, d, dims, splits > 1 ? ws.partial : nullptr, splits, kps, BN,
+                       stages, err));
   if (splits > 1) {
     const long long work = (long long)d.M * (d.N / 8);
     GCNN_TRY(launch(tc_reduce_kernel, ceil_div(work, 256), 256, 0, s, d, dims, (const float *)ws.partial, splits));

@@ -806,25 +806,26 @@ colsum_kernel(int n_cap, int cols0, int cols, DevDims dims, const float *__restr
     const float *src = first ? a0 + c : a1 + (c - cols0);
     const int ld = first ? ld0 : ld1;
     const float *mk = first ? mask : nullptr;
+    // every load of a pass before any use: rows past the range repeat its
+    // last one and are not added
     for (int i = i0 + (threadIdx.x >> 3); i < i1; i += 4 * kRowsPerPass) {
-      float4 x[4];
+      float4 x[4], m[4];
 #pragma unroll
       for (int u = 0; u < 4; ++u) {
-        const int r = i + u * kRowsPerPass;
-        if (r < i1) {
-          x[u] = ld4(src + (size_t)r * ld);
-          if (mk) {
-            const float4 m = ld4(mk + (size_t)r * ldm + c);
-            x[u].x = m.x > 0.f ? x[u].x : 0.f;
-            x[u].y = m.y > 0.f ? x[u].y : 0.f;
-            x[u].z = m.z > 0.f ? x[u].z : 0.f;
-            x[u].w = m.w > 0.f ? x[u].w : 0.f;
-          }
-        }
+        const size_t r = (size_t)min(i + u * kRowsPerPass, i1 - 1);
+        x[u] = ld4(src + r * ld);
+        if (mk) m[u] = ld4(mk + r * ldm + c);
       }
 #pragma unroll
-      for (int u = 0; u < 4; ++u)
+      for (int u = 0; u < 4; ++u) {
+        if (mk) {
+          x[u].x = m[u].x > 0.f ? x[u].x : 0.f;
+          x[u].y = m[u].y > 0.f ? x[u].y : 0.f;
+          x[u].z = m[u].z > 0.f ? x[u].z : 0.f;
+          x[u].w = m[u].w > 0.f ? x[u].w : 0.f;
+        }
         if (i + u * kRowsPerPass < i1) acc = add4(acc, x[u]);
+      }
     }
   }
 #pragma unroll
@@ -926,7 +927,6 @@ int launch_pool_bwd(int G, int n_nodes, int H, DevDims dims, const int *node_off
 
 namespace {
 constexpr int kHeadSmemFloats = 40 * 1024;  // 160 KB: W1 rows plus pooled / z1 / dz1 vectors
-
 constexpr size_t kHeadForwardBytes = 224 * 1024;
 
 // W1 in one chunk, in whole float4 columns
@@ -935,6 +935,7 @@ bool head_one_chunk(const HeadArgs &a) { return a.rk >= a.H && a.Hh % 4 == 0; }
 size_t head_forward_bytes(const HeadArgs &a) {
   return sizeof(float) * (size_t)a.H * a.Hh + sizeof(float4) * ((size_t)a.H + kHeadBatch * kHeadRed);
 }
+
 template <bool F, bool B>
 int head_graph(HeadArgs a, cudaStream_t s) {
   static bool configured = false;

@@ -21,6 +21,7 @@
 #include <mutex>
 
 #include "kernels.cuh"
+#include "slices.cuh"
 
 namespace gcnn {
 namespace {
@@ -247,6 +248,95 @@ aggregate_fwd_kernel(int n_cap, int H, DevDims dims, const int *__restrict__ row
 #pragma unroll
       for (int a = 0; a < kAgg; ++a)
         st_bf16x4(o + (q * kAgg + a) * H, sc[q] * vv[a].x, sc[q] * vv[a].y, sc[q] * vv[a].z, sc[q] * vv[a].w);
+  }
+}
+
+// The forward's aggregates of one node as integer slices for the tensor cores
+// (FP32 inference): a warp per node (H <= 256: two float4 columns per lane), so
+// that the row's largest magnitude is known before anything is written and the
+// FP32 aggregates never go to memory.  Rows with an infinity or a NaN get a NaN
+// factor and their FP32 aggregates, which the product then reads.
+constexpr int kSliceWarps = 4;
+
+__global__ void __launch_bounds__(32 * kSliceWarps)
+aggregate_slices_kernel(int n_cap, int H, int Ap, DevDims dims, const int *__restrict__ row_ptr,
+                        const int *__restrict__ col, const float *__restrict__ PQ, float *__restrict__ agg,
+                        uint16_t *__restrict__ agg3, float *__restrict__ factor, float eps,
+                        const unsigned *__restrict__ bad_weights, unsigned *err) {
+  pdl_entry(GCNN_K_AGG_FWD);
+  const int N = min(n_cap, dims.nodes(n_cap)), H4 = H >> 2;
+  const int i = blockIdx.x * kSliceWarps + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+  if (i >= N) return;  // warp-uniform
+  const int r0 = row_ptr[i], r1 = row_ptr[i + 1], d = r1 - r0;
+  if (d < 0 || r0 < 0) flag(err, kErrIndex);
+  const bool row = d > 0 && r0 >= 0;
+  int j[kCache];
+#pragma unroll
+  for (int k = 0; k < kCache; ++k) j[k] = row ? col[min(r0 + k, r1 - 1)] : i;
+  const float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
+  const Bonds none{nullptr, nullptr, 0};
+  const float df = (float)d;
+  float4 a[2][kAgg], P[2], first[2][kCache];
+  float m = 0.f;
+  // both columns' loads before any arithmetic
+#pragma unroll
+  for (int u = 0; u < 2; ++u) {
+    const int c = 4 * (lane + 32 * u);
+    if (!row || c >= H) continue;
+    P[u] = ld4(PQ + (size_t)i * 2 * H + c);
+    if (gather_first<false>(PQ, j, i, N, H, c, P[u], first[u], none, r0, r1)) flag(err, kErrIndex);
+  }
+#pragma unroll
+  for (int u = 0; u < 2; ++u) {
+    const int c = 4 * (lane + 32 * u);
+#pragma unroll
+    for (int q = 0; q < kAgg; ++q) a[u][q] = z;
+    if (!row || c >= H) continue;
+    const float4(&mc)[kCache] = first[u];
+    float4 s = z;
+    float4 mn = make_float4(FLT_MAX, FLT_MAX, FLT_MAX, FLT_MAX);
+    float4 mx = make_float4(-FLT_MAX, -FLT_MAX, -FLT_MAX, -FLT_MAX);
+    auto take = [&](float4 v) {
+      s = add4(s, v);
+      mn.x = fminf(mn.x, v.x); mn.y = fminf(mn.y, v.y); mn.z = fminf(mn.z, v.z); mn.w = fminf(mn.w, v.w);
+      mx.x = fmaxf(mx.x, v.x); mx.y = fmaxf(mx.y, v.y); mx.z = fmaxf(mx.z, v.z); mx.w = fmaxf(mx.w, v.w);
+    };
+#pragma unroll
+    for (int k = 0; k < kCache; ++k)
+      if (k < d) take(mc[k]);
+    for (int e = r0 + kCache; e < r1; ++e) take(message<false>(PQ, source(col, e, N, err), H, c, P[u], none, e));
+    const float4 mean = div_count(s, df);
+    float4 v = z;
+#pragma unroll
+    for (int k = 0; k < kCache; ++k)
+      if (k < d) acc_sq(v, mc[k], mean);
+    for (int e = r0 + kCache; e < r1; ++e)
+      acc_sq(v, message<false>(PQ, source(col, e, N, err), H, c, P[u], none, e), mean);
+    v = div_count(v, df);
+    a[u][0] = s;
+    a[u][1] = mean;
+    a[u][2] = mn;
+    a[u][3] = mx;
+    a[u][4] = make_float4(sqrtf(fmaxf(v.x, 0.f) + eps), sqrtf(fmaxf(v.y, 0.f) + eps), sqrtf(fmaxf(v.z, 0.f) + eps),
+                          sqrtf(fmaxf(v.w, 0.f) + eps));
+#pragma unroll
+    for (int q = 0; q < kAgg; ++q) m = max4(m, a[u][q]);
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+  float inv, f;
+  slice_scale(m, &inv, &f);
+  if (lane == 0) factor[i] = f;
+  const bool plain = bad_weights[0] != 0u;
+#pragma unroll
+  for (int u = 0; u < 2; ++u) {
+    const int c4 = lane + 32 * u;
+    if (c4 >= H4) continue;
+#pragma unroll
+    for (int q = 0; q < kAgg; ++q) {
+      if (f == f) store_slices(a[u][q], inv, agg3 + (size_t)i * 3 * Ap + q * H + 4 * c4, Ap);
+      if (f != f || plain) st4(agg + (size_t)i * kAgg * H + q * H + 4 * c4, a[u][q]);
+    }
   }
 }
 
@@ -623,6 +713,15 @@ int launch_aggregate_fwd(int n_nodes, int H, DevDims dims, const int *row_ptr, c
   GCNN_TRY(launch(kernel, ceil_div(work, kThreads), kThreads, 0, s, n_nodes, H, dims, row_ptr, col, PQ, agg, eps, err,
                   S16, ld16, amp, att, Bonds{eattr, wE, F}, idx_early ? 1 : 0));
   return GCNN_OK;
+}
+
+int launch_aggregate_slices(int n_nodes, int H, int Ap, DevDims dims, const int *row_ptr, const int *col,
+                            const float *PQ, float *agg, uint16_t *agg3, float *factor, float eps,
+                            const unsigned *bad_weights, unsigned *err, cudaStream_t s) {
+  if (H <= 0 || H % 4 || H > kF32MaxH) return set_error(GCNN_EINVAL, "aggregate: hidden out of range");
+  if (n_nodes <= 0) return GCNN_OK;
+  return launch(aggregate_slices_kernel, ceil_div(n_nodes, kSliceWarps), 32 * kSliceWarps, 0, s, n_nodes, H, Ap, dims,
+                row_ptr, col, PQ, agg, agg3, factor, eps, bad_weights, err);
 }
 
 int launch_aggregate_bwd(int n_nodes, int n_edges, int H, DevDims dims, const int *row_ptr,

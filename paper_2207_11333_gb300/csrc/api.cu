@@ -28,6 +28,7 @@ int timeline_attach_all(void *tl) {
   GCNN_TRY(timeline_attach_small(tl));
   GCNN_TRY(timeline_attach_gemm_simt(tl));
   GCNN_TRY(timeline_attach_gemm_tc(tl));
+  GCNN_TRY(timeline_attach_gemm_f32tc(tl));
   return GCNN_OK;
 }
 
@@ -123,6 +124,7 @@ void destroy_ctx(gcnn_ctx *c) {
   if (c->opt_ev) cudaEventDestroy(c->opt_ev);
   for (cudaEvent_t e : c->side_ev) cudaEventDestroy(e);
   if (c->order_dev) cudaFree(c->order_dev);
+  if (c->f32_mem) cudaFree(c->f32_mem);
   if (c->dmem) cudaFree(c->dmem);
   delete c;
 }
@@ -436,6 +438,7 @@ static int refresh_bf16(gcnn_ctx *c) {
 int gcnn_set_params(gcnn_ctx *c, const float *src, int64_t n, int on_device) {
   if (!src) return set_error(GCNN_EINVAL, "null source");
   GCNN_TRY(copy_flat(c, c ? c->params : nullptr, src, nullptr, n, on_device));
+  c->w3_stale = true;
   return refresh_bf16(c);
 }
 int gcnn_get_params(gcnn_ctx *c, float *dst, int64_t n, int on_device) {
@@ -486,6 +489,7 @@ int gcnn_load(gcnn_ctx *c, const char *path) {
             fread(buf.data(), sizeof(float), buf.size(), f) == buf.size();
   fclose(f);
   if (!ok) return set_error(GCNN_EFORMAT, "%s is not a checkpoint of this model", path);
+  c->w3_stale = true;
   GCNN_CUDA_TRY(cudaMemcpyAsync(c->params, buf.data(), c->P * sizeof(float), cudaMemcpyHostToDevice, c->stream));
   GCNN_CUDA_TRY(cudaMemcpyAsync(c->adam_m, buf.data() + c->P, c->P * sizeof(float), cudaMemcpyHostToDevice, c->stream));
   GCNN_CUDA_TRY(cudaMemcpyAsync(c->adam_v, buf.data() + 2 * c->P, c->P * sizeof(float), cudaMemcpyHostToDevice, c->stream));
@@ -570,7 +574,16 @@ int gcnn_forward(gcnn_ctx *c, const gcnn_batch *b, float *pred, int train) {
   if (!c) return set_error(GCNN_EINVAL, "null context");
   GCNN_TRY(same_batch(c, b));
   // same grid buckets as the captured step, so both give bit-identical results
-  GCNN_TRY(ctx_forward(c, b->n_graphs, grid_nodes(c, b), grid_edges(c, b), train != 0));
+  // FP32 inference on the tensor cores; not in a caller's own stream capture,
+  // whose replays have to follow later changes of the parameters
+  bool f32tc = !train && b->n_nodes > 0 && f32tc_wanted(c, grid_nodes(c, b));
+  if (f32tc) {
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    GCNN_CUDA_TRY(cudaStreamIsCapturing(c->stream, &cs));
+    if (cs != cudaStreamCaptureStatusNone) f32tc = false;
+    else GCNN_TRY(f32tc_prepare(c));
+  }
+  GCNN_TRY(ctx_forward(c, b->n_graphs, grid_nodes(c, b), grid_edges(c, b), train != 0, f32tc));
   if (pred && b->n_graphs > 0)
     GCNN_CUDA_TRY(cudaMemcpyAsync(pred, c->pred, b->n_graphs * sizeof(float), cudaMemcpyDeviceToDevice, c->stream));
   c->have_fwd = train != 0;
@@ -643,6 +656,7 @@ int gcnn_grads_device(gcnn_ctx *c, float **grads) {
 int gcnn_step(gcnn_ctx *c, float lr) {
   if (!c) return set_error(GCNN_EINVAL, "null context");
   GCNN_TRY(set_lr(c, lr));
+  c->w3_stale = true;
   return ctx_step(c);
 }
 
@@ -764,6 +778,7 @@ int run_step_graph(gcnn_ctx *c, const gcnn_batch *b, double *loss_accum, bool wi
     entry.range_ids = range_ids;
     it = c->graphs.emplace(key, std::move(entry)).first;
   }
+  if (with_step) c->w3_stale = true;
   GCNN_CUDA_TRY(cudaGraphLaunch(it->second.exec, c->stream));
   bool tl_on;
   {

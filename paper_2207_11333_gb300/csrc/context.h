@@ -69,6 +69,16 @@ struct gcnn_ctx {
   gcnn::GemmWorkspace ws{};
   gcnn::GemmWorkspace ws_side{};  // split-K partials of the GEMMs on the side stream
 
+  // FP32 inference on the tensor cores (f32tc_prepare): slices of x, the
+  // aggregates and the weights with their factors, and the update's phase values,
+  // in one allocation of its own, made on first use
+  char *f32_mem = nullptr;
+  uint16_t *x3 = nullptr, *agg3 = nullptr, *wm3 = nullptr, *wu3 = nullptr;
+  float *fx = nullptr, *fagg = nullptr, *fwm = nullptr, *fwu = nullptr, *f32_part = nullptr;
+  size_t f32_part_floats = 0;
+  unsigned *f32_bad = nullptr;  // a weight column without a finite factor
+  bool w3_stale = true;         // the parameters changed since the weights were sliced
+
   // host-side state
   bool have_fwd = false;
   int fwd_G = 0, fwd_N = 0, fwd_E = 0;
@@ -139,7 +149,13 @@ int ctx_range_prepare(gcnn_ctx *c, const gcnn_store *st, int64_t first, int32_t 
 int ctx_range_launch(gcnn_ctx *c, const gcnn_store *st, int64_t first, int32_t count);
 int ctx_range_update(gcnn_ctx *c, const gcnn_store *st, int64_t first, int32_t count, cudaGraphExec_t exec,
                      cudaGraphNode_t scan_node, cudaGraphNode_t graph_node);
-int ctx_forward(gcnn_ctx *c, int G, int Ngrid, int Egrid, bool train);
+// f32tc: the inference forward with f32tc_prepare done
+int ctx_forward(gcnn_ctx *c, int G, int Ngrid, int Egrid, bool train, bool f32tc = false);
+// Whether an inference forward over Ngrid nodes runs its FP32 products on the
+// tensor cores, and what that needs: buffers on first use (allocates) and the
+// weights' slices when the parameters changed (launches on the stream).
+bool f32tc_wanted(const gcnn_ctx *c, int Ngrid);
+int f32tc_prepare(gcnn_ctx *c);
 int ctx_backward(gcnn_ctx *c, int G, int Ngrid, int Egrid, const float *dpred, double *loss_accum);
 int ctx_step(gcnn_ctx *c);
 }  // namespace gcnn

@@ -299,6 +299,50 @@ int launch_pack_layer(int H, const float *msg_w, const float *upd_w, uint16_t *W
 int launch_colsum2(int n_cap, int cols0, int cols1, DevDims dims, const float *a0, int ld0, const float *mask,
                    int ldm, const float *a1, int ld1, float *out0, float *out1, cudaStream_t s);
 
+// ---------------------------------------------------------------- gemm_f32tc.cu
+// FP32 products of the inference forward on the tensor cores through exact
+// integer slices (described in the source).  A row's slices lie in one row of
+// three planes, each Hp (x) or Ap (aggregates) columns wide, a multiple of 64
+// whose padding stays zero; its factor is the power of two that scales them.
+constexpr int kF32Phases = 4, kF32MaxH = 256;
+struct F32Phase {
+  int from_agg;         // A: 0 the rows of x, 1 the aggregates
+  int b_row;            // first row of this phase's block of W
+  int ktiles;           // 64-wide k tiles
+  const float *scaler;  // per-node factor of the phase's value, or nullptr
+};
+struct F32Desc {
+  int M, N;
+  int nphase;
+  F32Phase phase[kF32Phases];  // the first without scaler; values are added in order
+  const uint16_t *x3, *agg3;
+  int Hp, Ap;
+  const float *fx, *fagg;      // row factors
+  const uint16_t *b3;          // three planes of b_rows x N
+  int b_rows;
+  const float *fb;             // column factors
+  float *C;
+  int ldc;
+  const float *bias;           // bias[n] for n < bias_n
+  int bias_n;
+  bool relu;
+  // FP32 operands, read where a factor is not finite (agg then holds the row)
+  const float *x, *agg, *W;
+  int H;
+};
+int run_gemm_f32tc(const F32Desc &d, DevDims dims, float *partial, size_t partial_floats, unsigned *err, cudaStream_t s);
+int launch_slice_rows(int n_nodes, int H, int Hp, DevDims dims, const float *x, uint16_t *x3, float *factor,
+                      cudaStream_t s);
+// count matrices of K x N, `stride` floats apart, into count x three K x N
+// planes; *bad (zeroed by the caller) is set where a column has no finite factor
+int launch_slice_weights(int K, int N, int count, const float *W, long long stride, uint16_t *w3, float *factor,
+                         unsigned *bad, cudaStream_t s);
+// The aggregates of launch_aggregate_fwd (no bond term) as slices.  Rows
+// without a finite factor, and every row where *bad_weights is set, go to agg.
+int launch_aggregate_slices(int n_nodes, int H, int Ap, DevDims dims, const int *row_ptr, const int *col,
+                            const float *PQ, float *agg, uint16_t *agg3, float *factor, float eps,
+                            const unsigned *bad_weights, unsigned *err, cudaStream_t s);
+
 // Timeline marker after a train step: records the end of the step's last kernel.
 int launch_step_end(cudaStream_t s);
 
@@ -311,5 +355,6 @@ int timeline_attach_aggregate(void *tl);
 int timeline_attach_small(void *tl);
 int timeline_attach_gemm_simt(void *tl);
 int timeline_attach_gemm_tc(void *tl);
+int timeline_attach_gemm_f32tc(void *tl);
 
 }  // namespace gcnn

@@ -465,7 +465,112 @@ PhaseScope::~PhaseScope() {
   else cudaEventRecord(c_->prof_ev[2 * idx_ + 1], c_->stream);
 }
 
-int ctx_forward(gcnn_ctx *c, int G, int Ngrid, int Egrid, bool train) {
+namespace {
+// Widths of the slices' planes: whole k tiles
+int plane_x(const gcnn_ctx *c) { return pad64(c->H); }
+int plane_agg(const gcnn_ctx *c) { return pad64(kAgg * c->H); }
+
+F32Desc f32_desc(gcnn_ctx *c, int Ngrid, int l) {
+  F32Desc d{};
+  d.M = Ngrid;
+  d.x3 = c->x3; d.agg3 = c->agg3; d.Hp = plane_x(c); d.Ap = plane_agg(c);
+  d.fx = c->fx; d.fagg = c->fagg;
+  d.x = xs_at(c, l); d.agg = agg_at(c, l); d.H = c->H;
+  return d;
+}
+
+// One layer of the FP32 inference forward on the tensor cores.
+int f32tc_layer(gcnn_ctx *c, int Ngrid, int l) {
+  const int H = c->H;
+  DevDims dims{c->bb.dims};
+  LayerW w = layer_ptrs(c->params, c, l);
+  const size_t part = c->f32_part_floats;
+  {
+    PhaseScope ps(c, GCNN_PHASE_GEMM);
+    GCNN_TRY(launch_slice_rows(Ngrid, H, plane_x(c), dims, xs_at(c, l), c->x3, c->fx, c->stream));
+    F32Desc d = f32_desc(c, Ngrid, l);  // PQ = x [A | B] + [b_M | 0]
+    d.N = 2 * H;
+    d.nphase = 1;
+    d.phase[0] = F32Phase{0, 0, d.Hp / 64, nullptr};
+    d.b3 = c->wm3 + (size_t)l * 3 * H * 2 * H; d.b_rows = H; d.fb = c->fwm + (size_t)l * 2 * H;
+    d.W = w.msg_w;
+    d.C = pq_at(c, l); d.ldc = 2 * H; d.bias = w.msg_b; d.bias_n = H;
+    GCNN_TRY(run_gemm_f32tc(d, dims, c->f32_part, part, c->err, c->stream));
+  }
+  {
+    PhaseScope ps(c, GCNN_PHASE_AGG_FWD);
+    GCNN_TRY(launch_aggregate_slices(Ngrid, H, plane_agg(c), dims, c->bb.row_ptr, c->bb.col, pq_at(c, l), agg_at(c, l),
+                                     c->agg3, c->fagg, (float)c->cfg.std_eps, c->f32_bad, c->err, c->stream));
+  }
+  PhaseScope ps(c, GCNN_PHASE_GEMM);
+  F32Desc d = f32_desc(c, Ngrid, l);  // x' = ReLU(x W_x + agg W_id + amp (agg W_amp) + att (agg W_att) + b_U)
+  d.N = H;
+  d.nphase = 4;
+  d.phase[0] = F32Phase{0, 0, d.Hp / 64, nullptr};
+  d.phase[1] = F32Phase{1, H, d.Ap / 64, nullptr};
+  d.phase[2] = F32Phase{1, 6 * H, d.Ap / 64, c->bb.amp};
+  d.phase[3] = F32Phase{1, 11 * H, d.Ap / 64, c->bb.att};
+  d.b3 = c->wu3 + (size_t)l * 3 * 16 * H * H; d.b_rows = 16 * H; d.fb = c->fwu + (size_t)l * H;
+  d.W = w.upd_w;
+  d.C = xs_at(c, l + 1); d.ldc = H; d.bias = w.upd_b; d.bias_n = H; d.relu = true;
+  return run_gemm_f32tc(d, dims, c->f32_part, part, c->err, c->stream);
+}
+}  // namespace
+
+// Widths from 64 (narrower rows fill the 64-wide k tiles badly) to what a warp
+// holds of a row, without bond features.  Row-invariant contexts take it at any
+// size, since a molecule's result may not depend on its batch-mates; others
+// from 2,048 rows, where it begins to win over split-K on the CUDA cores.
+bool f32tc_wanted(const gcnn_ctx *c, int Ngrid) {
+  return c->cfg.precision == GCNN_PREC_FP32 && c->cfg.edge_features == 0 && c->H >= 64 && c->H <= kF32MaxH &&
+         ((c->cfg.flags & GCNN_FLAG_ROW_INVARIANT) || Ngrid >= 2048);
+}
+
+int f32tc_prepare(gcnn_ctx *c) {
+  const size_t H = c->H, L = c->L, N = c->Nc;
+  if (!c->f32_mem) {
+    size_t off = 0;
+    auto take = [&off](size_t bytes) {
+      const size_t at = off;
+      off = (off + bytes + 255) / 256 * 256;
+      return at;
+    };
+    // phase values: up to 20,480 rows run their phases in parallel CTAs
+    const size_t part = 4 * std::min<size_t>(N, 20480) * H;
+    const size_t o_x = take(2 * N * 3 * plane_x(c)), o_a = take(2 * N * 3 * plane_agg(c));
+    const size_t o_wm = take(2 * L * 3 * H * 2 * H), o_wu = take(2 * L * 3 * 16 * H * H);
+    const size_t o_fx = take(4 * N), o_fa = take(4 * N), o_fm = take(4 * L * 2 * H), o_fu = take(4 * L * H);
+    const size_t o_p = take(4 * part), o_bad = take(4);
+    char *m = nullptr;
+    const cudaError_t e = cudaMalloc(&m, off);
+    if (e != cudaSuccess) return set_error(GCNN_ENOMEM, "cudaMalloc(%zu bytes): %s", off, cudaGetErrorString(e));
+    // the planes' padding stays zero
+    const cudaError_t z = cudaMemsetAsync(m, 0, off, c->stream);
+    if (z != cudaSuccess) {
+      cudaFree(m);
+      return set_error(GCNN_ECUDA, "cudaMemset: %s", cudaGetErrorString(z));
+    }
+    c->f32_mem = m;
+    c->x3 = (uint16_t *)(m + o_x); c->agg3 = (uint16_t *)(m + o_a);
+    c->wm3 = (uint16_t *)(m + o_wm); c->wu3 = (uint16_t *)(m + o_wu);
+    c->fx = (float *)(m + o_fx); c->fagg = (float *)(m + o_fa);
+    c->fwm = (float *)(m + o_fm); c->fwu = (float *)(m + o_fu);
+    c->f32_part = (float *)(m + o_p); c->f32_part_floats = part;
+    c->f32_bad = (unsigned *)(m + o_bad);
+    c->dbytes += off;
+    c->w3_stale = true;
+  }
+  if (c->w3_stale) {
+    LayerW w = layer_ptrs(c->params, c, 0);
+    GCNN_CUDA_TRY(cudaMemsetAsync(c->f32_bad, 0, sizeof(unsigned), c->stream));
+    GCNN_TRY(launch_slice_weights(c->H, 2 * c->H, c->L, w.msg_w, c->layer_size, c->wm3, c->fwm, c->f32_bad, c->stream));
+    GCNN_TRY(launch_slice_weights(16 * c->H, c->H, c->L, w.upd_w, c->layer_size, c->wu3, c->fwu, c->f32_bad, c->stream));
+    c->w3_stale = false;
+  }
+  return GCNN_OK;
+}
+
+int ctx_forward(gcnn_ctx *c, int G, int Ngrid, int Egrid, bool train, bool f32tc) {
   (void)Egrid;
   const int H = c->H;
   DevDims dims{c->bb.dims};
@@ -476,6 +581,10 @@ int ctx_forward(gcnn_ctx *c, int G, int Ngrid, int Egrid, bool train) {
                           bf ? X_at(c, 0) : nullptr, X_ld(c)));
   }
   for (int l = 0; l < c->L; ++l) {
+    if (f32tc) {
+      GCNN_TRY(f32tc_layer(c, Ngrid, l));
+      continue;
+    }
     if (bf) GCNN_TRY(tc_message(c, Ngrid, l));
     else GCNN_TRY(gemm_message(c, Ngrid, l));
     {

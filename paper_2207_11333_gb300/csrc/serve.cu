@@ -156,7 +156,7 @@ int capture_forward(gcnn_ctx *c, int G, int Ngrid, int Egrid, cudaGraphExec_t *o
   c->stream = c->cap_stream;
   c->capturing = true;
   cudaError_t e = cudaStreamBeginCapture(c->stream, cudaStreamCaptureModeThreadLocal);
-  int rc = e == cudaSuccess ? ctx_forward(c, G, Ngrid, Egrid, false)
+  int rc = e == cudaSuccess ? ctx_forward(c, G, Ngrid, Egrid, false, f32tc_wanted(c, Ngrid))
                             : set_error(GCNN_ECUDA, "begin capture: %s", cudaGetErrorString(e));
   if (e == cudaSuccess) {
     cudaError_t e2 = cudaStreamEndCapture(c->stream, &graph);
@@ -452,6 +452,11 @@ int gcnn_serve_create(const gcnn_ctx *model, const gcnn_serve_config *cfg, gcnn_
     rc = gcnn_create(&sc, sl.stream, &sl.ctx);
     if (rc != GCNN_OK) break;
     rc = gcnn_set_params(sl.ctx, model->params, sl.ctx->P, 1);
+    if (rc != GCNN_OK) break;
+    // the slots' parameters never change: their slices are made once
+    if (f32tc_wanted(sl.ctx, max_nodes)) rc = f32tc_prepare(sl.ctx);
+    if (rc == GCNN_OK && cudaStreamSynchronize(sl.stream) != cudaSuccess)
+      rc = set_error(GCNN_ECUDA, "serve_create: cannot prepare a slot");
     if (rc != GCNN_OK) break;
     // every bucket's forward graph is captured now, so that no request
     // waits for a capture

@@ -310,8 +310,14 @@ void retire(gcnn_server *s, Slot &sl) {
   s->done_cv.notify_all();
 }
 
+// A small batch takes about 150 us on the device, no more than a sleeping
+// thread needs to be woken twice: after it last had something to do the
+// scheduler looks on for this long before it sleeps.
+constexpr auto kSpin = std::chrono::microseconds(300);
+
 void worker_loop(gcnn_server *s) {
   cudaSetDevice(s->device);
+  auto active = Clock::now();
   for (;;) {
     bool progressed = false;
     for (Slot &sl : s->slots) {
@@ -356,13 +362,18 @@ void worker_loop(gcnn_server *s) {
     bool any_busy = false;
     for (Slot &sl : s->slots) any_busy |= sl.busy;
     if (s->stop.load() && !any_busy) break;
-    if (!progressed) {
+    if (progressed) {
+      active = Clock::now();
+    } else if (Clock::now() - active < kSpin) {
+      std::this_thread::yield();
+    } else {
       if (any_busy) {
         std::this_thread::sleep_for(std::chrono::microseconds(20));
       } else {
         std::unique_lock<std::mutex> lock(s->mu);
         s->work_cv.wait_for(lock, std::chrono::milliseconds(2),
                             [s] { return s->stop.load() || (!s->pending.empty() && s->fatal == GCNN_OK); });
+        if (!s->pending.empty()) active = Clock::now();
       }
     }
   }

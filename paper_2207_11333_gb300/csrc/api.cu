@@ -373,7 +373,7 @@ int gcnn_create(const gcnn_config *cfg, void *stream, gcnn_ctx **out) {
         cudaStreamCreateWithFlags(&c->opt, cudaStreamNonBlocking) != cudaSuccess ||
         cudaEventCreateWithFlags(&c->opt_ev, cudaEventDisableTiming) != cudaSuccess)
       rc = set_error(GCNN_ECUDA, "cannot create the side streams");
-    for (int q = 0; q < 3 * c->L + 1 && rc == GCNN_OK; ++q) {
+    for (int q = 0; q < 4 * c->L + 1 && rc == GCNN_OK; ++q) {
       cudaEvent_t ev = nullptr;
       if (cudaEventCreateWithFlags(&ev, cudaEventDisableTiming) != cudaSuccess)
         rc = set_error(GCNN_ECUDA, "cannot create events");

@@ -13,8 +13,10 @@ struct gcnn_ctx {
   cudaStream_t cap_stream = nullptr;  // private stream used only for graph capture
   cudaStream_t side = nullptr;        // BF16 backward: weight-gradient work off the critical path
   std::vector<cudaEvent_t> side_ev;   // 3 per layer: fork, aggregate gradient done, side work done;
-                                      // then one for the head gradients
-  cudaStream_t opt = nullptr;         // train step: early AdamW updates of layers L-1 .. 1
+                                      // then one for the head gradients, then the
+                                      // bond rows' gradients done, 1 per layer
+  cudaStream_t opt = nullptr;         // train step: early AdamW updates of layers L-1 .. 1;
+                                      // overlapped backward: bond rows' gradients
   cudaEvent_t opt_ev = nullptr;       // their completion
   int device = 0;
   int H = 0, L = 0, T = 0, Hh = 0;

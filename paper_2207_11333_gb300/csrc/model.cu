@@ -118,10 +118,10 @@ int gemm(gcnn_ctx *c, const GemmDesc &d) {
 // each edge's message gradient at its reverse slot, and both directions of a
 // bond carry the same features (checked when the store is opened), so slot r
 // pairs dm[r] with eattr[r].
-int gemm_bond_rows(gcnn_ctx *c, int Egrid, float *g_edge_w) {
+int gemm_bond_rows(gcnn_ctx *c, int Egrid, float *g_edge_w, cudaStream_t s) {
   PhaseScope ps(c, GCNN_PHASE_AGG_BWD);
   return launch_bond_grad(Egrid, c->H, c->cfg.edge_features, c->bb.eattr_ld, DevDims{c->bb.dims}, c->bb.eattr, c->dm,
-                          g_edge_w, c->stream);
+                          g_edge_w, s);
 }
 
 // Node-level head forward on the last layer (zn = x W1n + b1n, then the
@@ -155,9 +155,17 @@ int node_head_forward(gcnn_ctx *c, int Ngrid, bool train) {
   return GCNN_OK;
 }
 
+// The stream (and split-K workspace) of a layer's weight- and bias-gradient
+// work: a second stream that overlaps the data-gradient chain, or the main
+// stream when the step runs serially.
+struct Lane {
+  cudaStream_t s;
+  const GemmWorkspace *ws;
+};
+
 // Node-level head parameter gradients: [x ; 1]^T dzn -> W1n and b1n, then
 // w2n, b2n and the node loss sums.
-int node_head_backward(gcnn_ctx *c, int Ngrid, double *loss_accum) {
+int node_head_backward(gcnn_ctx *c, int Ngrid, double *loss_accum, Lane lane) {
   const int H = c->H, Hh = c->Hh;
   float *gw = node_head_ptr(c->grads, c);
   GemmDesc d = blank();
@@ -168,9 +176,12 @@ int node_head_backward(gcnn_ctx *c, int Ngrid, double *loss_accum) {
   d.A.seg[1] = seg(H, nullptr, 0);
   d.B.nseg = 1; d.B.seg[0] = seg(0, c->dzn, Hh);
   d.C = gw; d.ldc = Hh;
-  GCNN_TRY(gemm(c, d));
+  {
+    PhaseScope ps(c, GCNN_PHASE_GEMM);
+    GCNN_TRY(run_gemm_simt(d, DevDims{c->bb.dims}, *lane.ws, lane.s));
+  }
   PhaseScope ps(c, GCNN_PHASE_HEAD);
-  GCNN_TRY(launch_node_grad(node_args(c, Ngrid), gw + (int64_t)H * Hh + Hh, loss_accum, c->stream));
+  GCNN_TRY(launch_node_grad(node_args(c, Ngrid), gw + (int64_t)H * Hh + Hh, loss_accum, lane.s));
   return GCNN_OK;
 }
 
@@ -178,14 +189,6 @@ int tc(gcnn_ctx *c, const TcDesc &d) {
   PhaseScope ps(c, GCNN_PHASE_GEMM);
   return run_gemm_tc(d, DevDims{c->bb.dims}, c->ws, c->err, c->stream);
 }
-
-// The stream (and split-K workspace) of a layer's weight- and bias-gradient
-// work: a second stream that overlaps the data-gradient chain, or the main
-// stream when the step runs serially.
-struct Lane {
-  cudaStream_t s;
-  const GemmWorkspace *ws;
-};
 
 int tc_on(gcnn_ctx *c, const TcDesc &d, Lane lane) {
   PhaseScope ps(c, GCNN_PHASE_GEMM);
@@ -310,6 +313,9 @@ int tc_update(gcnn_ctx *c, int Ngrid, int l) {
   return tc(c, d);
 }
 
+// Completion of the bond rows' gradient of layer l (overlapped backward)
+cudaEvent_t bond_event(const gcnn_ctx *c, int l) { return c->side_ev[3 * c->L + 1 + l]; }
+
 // BF16 backward of layer l.  dH holds dL/dx_{l+1} (FP32) and G5[cur] its
 // masked, scaled BF16 form in columns [0, 3H).  Writes dX = dL/dx_l and, for
 // l > 0, columns [0, 3H) of G5[cur ^ 1]; [dP | dQ] goes to dPQ (FP32) and to
@@ -379,6 +385,8 @@ int tc_backward_layer(gcnn_ctx *c, int Gn, int Ngrid, int Egrid, int l, int cur,
   }
   {
     PhaseScope ps(c, GCNN_PHASE_AGG_BWD);
+    // dm is free once the bond rows of the layer above have read it
+    if (ov && c->cfg.edge_features > 0 && l + 1 < c->L) GCNN_CUDA_TRY(cudaStreamWaitEvent(c->stream, bond_event(c, l + 1), 0));
     // layers run from L - 1 down: the first one cuts the batch into chunks, the rest reuse them
     GCNN_TRY(launch_aggregate_bwd_graphs(Gn, Ngrid, Egrid, H, dims, c->bb.node_off, c->bb.row_ptr, c->bb.col,
                                          c->bb.rev, pq, agg, c->dagg, dPQ, c->dm, c->chunks,
@@ -386,11 +394,17 @@ int tc_backward_layer(gcnn_ctx *c, int Gn, int Ngrid, int Egrid, int l, int cur,
                                          layer_ptrs(c->params, c, l).edge_w, c->cfg.edge_features,
                                          l == c->L - 1, true));
   }
-  // before the next layer's aggregation backward reuses dm
-  if (c->cfg.edge_features > 0) GCNN_TRY(gemm_bond_rows(c, Egrid, gw.edge_w));
+  if (c->cfg.edge_features > 0 && !ov) GCNN_TRY(gemm_bond_rows(c, Egrid, gw.edge_w, c->stream));
   if (ov) {
     GCNN_CUDA_TRY(cudaEventRecord(mid, c->stream));
     GCNN_CUDA_TRY(cudaStreamWaitEvent(lane.s, mid, 0));
+    // the bond rows' gradient on the third stream, beside the dx and dagg GEMMs:
+    // in the chain itself it cost 15 us a layer
+    if (c->cfg.edge_features > 0) {
+      GCNN_CUDA_TRY(cudaStreamWaitEvent(c->opt, mid, 0));
+      GCNN_TRY(gemm_bond_rows(c, Egrid, gw.edge_w, c->opt));
+      GCNN_CUDA_TRY(cudaEventRecord(bond_event(c, l), c->opt));
+    }
   }
   {  // dW_M = x^T [dP | dQ]
     TcDesc d = tblank();
@@ -606,22 +620,25 @@ int ctx_forward(gcnn_ctx *c, int G, int Ngrid, int Egrid, bool train, bool f32tc
 int ctx_backward(gcnn_ctx *c, int G, int Ngrid, int Egrid, const float *dpred, double *loss_accum) {
   const int H = c->H;
   DevDims dims{c->bb.dims};
-  if (c->cfg.node_head) GCNN_TRY(node_head_backward(c, Ngrid, loss_accum));
+  // the heads' parameter gradients and loss sums feed only the optimiser: on
+  // the side lane when the backward overlaps
+  const bool heads_aside = bf16(c) && overlapped(c);
+  if (c->cfg.node_head && !heads_aside) GCNN_TRY(node_head_backward(c, Ngrid, loss_accum, Lane{c->stream, &c->ws}));
   {
     PhaseScope ps(c, GCNN_PHASE_HEAD);
     if (!c->fuse_head) GCNN_TRY(launch_head_graph(head_args(c, G, dpred), false, true, c->stream));
     HeadGradArgs ga{G, H, c->Hh, dims, c->pooled, c->z1, c->dz1, c->dpred, c->pred, c->bb.y,
                     head_ptr(c->grads, c), loss_accum};
-    // the head's parameter gradients and loss sums feed only the optimiser:
-    // on the side lane when the backward overlaps
     cudaStream_t hs = c->stream;
-    if (bf16(c) && overlapped(c)) {
+    if (heads_aside) {
       cudaEvent_t ev = c->side_ev[3 * c->L];
       GCNN_CUDA_TRY(cudaEventRecord(ev, c->stream));
       GCNN_CUDA_TRY(cudaStreamWaitEvent(c->side, ev, 0));
       hs = c->side;
     }
     GCNN_TRY(launch_head_grad(ga, hs));
+    if (c->cfg.node_head && heads_aside)
+      GCNN_TRY(node_head_backward(c, Ngrid, loss_accum, Lane{c->side, &c->ws_side}));
   }
   if (bf16(c)) {
     const bool ov = overlapped(c);
@@ -685,7 +702,7 @@ int ctx_backward(gcnn_ctx *c, int G, int Ngrid, int Egrid, const float *dpred, d
                                            (float)c->cfg.std_eps, c->err, c->stream, nullptr, 0, c->bb.eattr,
                                            w.edge_w, c->cfg.edge_features, l == c->L - 1, true));
     }
-    if (c->cfg.edge_features > 0) GCNN_TRY(gemm_bond_rows(c, Egrid, gw.edge_w));
+    if (c->cfg.edge_features > 0) GCNN_TRY(gemm_bond_rows(c, Egrid, gw.edge_w, c->stream));
     // dW_M (H x 2H) and db_M: [x ; 1]^T dPQ  (bias row keeps the first H columns)
     {
       GemmDesc d = blank();
@@ -726,6 +743,7 @@ int ctx_backward(gcnn_ctx *c, int G, int Ngrid, int Egrid, const float *dpred, d
     // gradients and the head's on the second stream, and the third stream's
     // updates join here
     GCNN_CUDA_TRY(cudaStreamWaitEvent(c->stream, c->side_ev[2], 0));
+    if (c->cfg.edge_features > 0) GCNN_CUDA_TRY(cudaStreamWaitEvent(c->stream, bond_event(c, 0), 0));
     if (layers_updated_early(c) && c->L >= 2) GCNN_CUDA_TRY(cudaStreamWaitEvent(c->stream, c->opt_ev, 0));
   }
   return mark_grads_ready(c, c->L, c->stream);  // every gradient is final here

@@ -655,8 +655,22 @@ __global__ void __launch_bounds__(kRedThreads) node_grad_kernel(NodeHeadArgs a, 
   if ((int)blockIdx.x < gridDim.x - 1) {
     const int c = blockIdx.x * 32 + lane;
     float s = 0.f;
+    // the loads of sixteen atoms in flight, added in order (atoms past the last
+    // one repeat it and are not added)
+    constexpr int U = 16, W = kRedThreads / 32;
     if (c < a.Hh)
-      for (int i = w; i < N; i += kRedThreads / 32) s += fmaxf(a.zn[(size_t)i * a.Hh + c], 0.f) * a.dpred[i];
+      for (int i = w; i < N; i += U * W) {
+        float z[U], d[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+          const size_t r = (size_t)min(i + u * W, N - 1);
+          z[u] = a.zn[r * a.Hh + c];
+          d[u] = a.dpred[r];
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+          if (i + u * W < N) s += fmaxf(z[u], 0.f) * d[u];
+      }
     part[w][lane] = s;
     __syncthreads();
     if (w == 0 && c < a.Hh) {

@@ -549,16 +549,30 @@ __global__ void __launch_bounds__(kRedThreads) head_grad_kernel(HeadGradArgs a) 
   if ((int)blockIdx.y < (H + kHT - 1) / kHT) {
     const int k0 = blockIdx.y * kHT;
     float acc[4] = {0.f, 0.f, 0.f, 0.f};
+    // the next kHG graphs' values travel in registers while these are used
+    constexpr int V = kHG * kHT / kRedThreads;
+    float rp[V], rd[V];
+    auto load = [&](int g0) {
+#pragma unroll
+      for (int v = 0; v < V; ++v) {
+        const int q = tid + v * kRedThreads, g = g0 + q / kHT, cc = q % kHT;
+        rp[v] = g < G && k0 + cc < H ? a.pooled[(size_t)g * H + k0 + cc] : 0.f;
+        rd[v] = g < G && c0 + cc < Hh ? a.dz1[(size_t)g * Hh + c0 + cc] : 0.f;
+      }
+    };
+    load(0);
     for (int g0 = 0; g0 < G; g0 += kHG) {
       const int gn = min(kHG, G - g0);
       __syncthreads();
-      for (int q = tid; q < kHG * kHT; q += kRedThreads) {
-        const int gg = q / kHT, cc = q % kHT;
-        const bool in = gg < gn;
-        sp[gg][cc] = in && k0 + cc < H ? a.pooled[(size_t)(g0 + gg) * H + k0 + cc] : 0.f;
-        sd[gg][cc] = in && c0 + cc < Hh ? a.dz1[(size_t)(g0 + gg) * Hh + c0 + cc] : 0.f;
+#pragma unroll
+      for (int v = 0; v < V; ++v) {
+        const int q = tid + v * kRedThreads;
+        sp[q / kHT][q % kHT] = rp[v];
+        sd[q / kHT][q % kHT] = rd[v];
       }
       __syncthreads();
+      if (g0 + kHG < G) load(g0 + kHG);
+#pragma unroll 8
       for (int gg = 0; gg < gn; ++gg) {
         const float d = sd[gg][tc];
 #pragma unroll
@@ -577,11 +591,26 @@ __global__ void __launch_bounds__(kRedThreads) head_grad_kernel(HeadGradArgs a) 
   // b1 and w2 for columns c0 .. c0 + 31: graphs strided over the 8 warps
   {
     const int c = c0 + tc;
+    // eight graphs' loads in flight, added in order (graphs past the last one
+    // repeat it and are not added); one at a time they were most of this kernel
     float sb = 0.f, sw = 0.f;
+    constexpr int U = 8, W = kRedThreads / 32;
     if (c < Hh)
-      for (int g = q8; g < G; g += kRedThreads / 32) {
-        sb += a.dz1[(size_t)g * Hh + c];
-        sw += fmaxf(a.z1[(size_t)g * Hh + c], 0.f) * a.dpred[g];
+      for (int g = q8; g < G; g += U * W) {
+        float dz[U], z[U], dp[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+          const size_t r = (size_t)min(g + u * W, G - 1);
+          dz[u] = a.dz1[r * Hh + c];
+          z[u] = a.z1[r * Hh + c];
+          dp[u] = a.dpred[r];
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+          if (g + u * W < G) {
+            sb += dz[u];
+            sw += fmaxf(z[u], 0.f) * dp[u];
+          }
       }
     sp[q8][tc] = sb;
     sd[q8][tc] = sw;

@@ -544,7 +544,7 @@ int gcnn_op_aggregate_bwd(int32_t n_nodes, int32_t n_edges, int32_t hidden, cons
  * graphs: node_off (device, n_graphs + 1 int32) gives each graph's first node,
  * and no edge may leave its graph (as after gcnn_collate).  Batches of at
  * least 2 x (SM count) x 128 edges run one fused kernel: the batch is cut into
- * chunks of about 128 edges of whole graphs, and each block keeps its chunk's
+ * chunks of about 64 edges of whole graphs, and each block keeps its chunk's
  * per-edge gradients in shared memory, so they never travel to device memory
  * (graphs too large for that use scratch).  Smaller batches run the kernel
  * pair of gcnn_op_aggregate_bwd.  scratch (device) holds

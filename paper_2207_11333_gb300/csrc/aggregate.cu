@@ -26,7 +26,9 @@
 namespace gcnn {
 namespace {
 
-constexpr int kThreads = 256;
+// Eight blocks of 128 threads hold as many warps as four of 256 and leave the
+// SM sooner (forward of 300,000 atoms, H = 200: 346 -> 331 us).
+constexpr int kThreads = 128;
 
 __device__ __forceinline__ float4 ld4(const float *p) { return *reinterpret_cast<const float4 *>(p); }
 __device__ __forceinline__ void flag(unsigned *err, unsigned bits) {
@@ -157,7 +159,7 @@ __device__ __forceinline__ void acc_sq(float4 &v, float4 m, float4 mean) {
 // F32 / B16: whether the FP32 aggregates / the BF16 scaled operand are
 // written (one instantiation per output set keeps the other's code out)
 template <bool F32, bool B16, bool EDGE>
-__global__ void __launch_bounds__(kThreads, 4)
+__global__ void __launch_bounds__(kThreads, 8)
 aggregate_fwd_kernel(int n_cap, int H, DevDims dims, const int *__restrict__ row_ptr,
                      const int *__restrict__ col, const float *__restrict__ PQ,
                      float *__restrict__ agg, float eps, unsigned *err, uint16_t *__restrict__ S16, int ld16,
@@ -516,8 +518,17 @@ aggregate_bwd_edge_kernel(int n_cap, int e_cap, int H, DevDims dims, const int *
 // waits at its barrier between the passes the other loads, and the last wave
 // is finer than with one block of 512 (18,000 atoms, H = 200: 71 -> 63 us).
 constexpr int kFusedThreads = 256;
-constexpr int kChunkEdges = 128;  // edges per chunk on average (one window)
-constexpr int kChunkSlots = 192;  // edges a chunk keeps in shared memory (more costs L1)
+// Chunks of about 64 edges keep a whole row of up to 228 channels in one block,
+// so that a node's index and row bounds are read once and not per channel slice
+// (300,000 atoms, H = 200, against chunks of 128 edges and 192 slots in two
+// slices: 742 -> 685 us; H = 256, which has two slices either way: the same).
+// Fewer slots (96) send more chunks to the scratch in memory (H = 256: 6%
+// slower), more of them (128) split the row again (841 us).
+constexpr int kChunkEdges = 64;   // edges per chunk on average (one window)
+constexpr int kChunkSlots = 112;  // edges a chunk keeps in shared memory (more costs L1)
+// Below this many edges per SM the edge + gather pair runs: it spreads a small
+// batch over more blocks.
+constexpr int kFusedEdges = 256;
 constexpr int kFusedSmem = 100 * 1024;  // shared-memory budget of one block: two blocks per SM
 
 // Work partition of the fused backward: chunk k holds the graphs whose first
@@ -765,7 +776,7 @@ int launch_aggregate_bwd(int n_nodes, int n_edges, int H, DevDims dims, const in
 int aggregate_chunk_capacity(int n_edges) { return ceil_div(std::max(n_edges, 1), kChunkEdges) + 1; }
 
 bool aggregate_bwd_uses_fused(int n_edges) {
-  return ceil_div(std::max(n_edges, 0), kChunkEdges) >= 2 * num_sms();
+  return ceil_div(std::max(n_edges, 0), kFusedEdges / 2) >= 2 * num_sms();
 }
 
 int launch_aggregate_bwd_graphs(int n_graphs, int n_nodes, int n_edges, int H, DevDims dims, const int *node_off,

@@ -73,7 +73,7 @@ int launch_aggregate_bwd(int n_nodes, int n_edges, int H, DevDims dims, const in
 
 // The same gradient for a batch of whole graphs (node_off: G + 1 offsets;
 // no edge leaves its graph).  Batches of at least 2 x SMs x 128 edges take the
-// fused kernel: chunks of graphs of about 128 edges, each handled by one block
+// fused kernel: chunks of graphs of about 64 edges, each handled by one block
 // that keeps its per-edge gradients in shared memory; `chunks` holds
 // aggregate_chunk_capacity(n_edges) ints.  Smaller batches, and batches
 // with bond features (whose weight gradient reads the per-edge gradients in

@@ -573,16 +573,17 @@ int gcnn_batch_export(gcnn_ctx *c, const gcnn_batch *b, int32_t *node_off, int32
 int gcnn_forward(gcnn_ctx *c, const gcnn_batch *b, float *pred, int train) {
   if (!c) return set_error(GCNN_EINVAL, "null context");
   GCNN_TRY(same_batch(c, b));
-  // same grid buckets as the captured step, so both give bit-identical results
-  // FP32 inference on the tensor cores; not in a caller's own stream capture,
-  // whose replays have to follow later changes of the parameters
+  // FP32 inference on the tensor cores; in a caller's own stream capture only
+  // once its buffers are there (a forward before the capture makes them)
   bool f32tc = !train && b->n_nodes > 0 && f32tc_wanted(c, grid_nodes(c, b));
   if (f32tc) {
     cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
     GCNN_CUDA_TRY(cudaStreamIsCapturing(c->stream, &cs));
-    if (cs != cudaStreamCaptureStatusNone) f32tc = false;
-    else GCNN_TRY(f32tc_prepare(c));
+    const bool capturing = cs != cudaStreamCaptureStatusNone;
+    if (!capturing || c->f32_mem) GCNN_TRY(f32tc_prepare(c, capturing));
+    f32tc = c->f32_mem != nullptr;
   }
+  // same grid buckets as the captured step, so both give bit-identical results
   GCNN_TRY(ctx_forward(c, b->n_graphs, grid_nodes(c, b), grid_edges(c, b), train != 0, f32tc));
   if (pred && b->n_graphs > 0)
     GCNN_CUDA_TRY(cudaMemcpyAsync(pred, c->pred, b->n_graphs * sizeof(float), cudaMemcpyDeviceToDevice, c->stream));

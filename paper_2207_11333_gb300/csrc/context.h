@@ -77,9 +77,10 @@ struct gcnn_ctx {
   char *f32_mem = nullptr;
   uint16_t *x3 = nullptr, *agg3 = nullptr, *wm3 = nullptr, *wu3 = nullptr;
   float *fx = nullptr, *fagg = nullptr, *fwm = nullptr, *fwu = nullptr, *f32_part = nullptr;
-  size_t f32_part_floats = 0;
+  size_t f32_part_floats = 0, f32_bytes = 0;
   unsigned *f32_bad = nullptr;  // a weight column without a finite factor
   bool w3_stale = true;         // the parameters changed since the weights were sliced
+  bool f32_off = false;         // no memory for those buffers: FP32 inference stays on the CUDA cores
 
   // host-side state
   bool have_fwd = false;
@@ -155,9 +156,15 @@ int ctx_range_update(gcnn_ctx *c, const gcnn_store *st, int64_t first, int32_t c
 int ctx_forward(gcnn_ctx *c, int G, int Ngrid, int Egrid, bool train, bool f32tc = false);
 // Whether an inference forward over Ngrid nodes runs its FP32 products on the
 // tensor cores, and what that needs: buffers on first use (allocates) and the
-// weights' slices when the parameters changed (launches on the stream).
+// weights' slices when the parameters changed (launches on the stream).  Where
+// the device has no room for the buffers, prepare returns GCNN_OK with f32_off
+// set, and from then on the context runs them on the CUDA cores, so that all its
+// forwards keep one arithmetic.  capturing: the stream belongs to a capture, so
+// nothing is allocated, and the slicing is captured too (replays follow the
+// parameters).
 bool f32tc_wanted(const gcnn_ctx *c, int Ngrid);
-int f32tc_prepare(gcnn_ctx *c);
+int f32tc_prepare(gcnn_ctx *c, bool capturing = false);
+void f32tc_release(gcnn_ctx *c);  // frees the buffers and sets f32_off
 int ctx_backward(gcnn_ctx *c, int G, int Ngrid, int Egrid, const float *dpred, double *loss_accum);
 int ctx_step(gcnn_ctx *c);
 }  // namespace gcnn

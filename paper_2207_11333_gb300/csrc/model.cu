@@ -536,11 +536,21 @@ int f32tc_layer(gcnn_ctx *c, int Ngrid, int l) {
 // size, since a molecule's result may not depend on its batch-mates; others
 // from 2,048 rows, where it begins to win over split-K on the CUDA cores.
 bool f32tc_wanted(const gcnn_ctx *c, int Ngrid) {
-  return c->cfg.precision == GCNN_PREC_FP32 && c->cfg.edge_features == 0 && c->H >= 64 && c->H <= kF32MaxH &&
+  return !c->f32_off && c->cfg.precision == GCNN_PREC_FP32 && c->cfg.edge_features == 0 && c->H >= 64 &&
+         c->H <= kF32MaxH &&
          ((c->cfg.flags & GCNN_FLAG_ROW_INVARIANT) || Ngrid >= 2048);
 }
 
-int f32tc_prepare(gcnn_ctx *c) {
+void f32tc_release(gcnn_ctx *c) {
+  if (c->f32_mem) {
+    cudaFree(c->f32_mem);
+    c->dbytes -= c->f32_bytes;
+  }
+  c->f32_mem = nullptr;
+  c->f32_off = true;
+}
+
+int f32tc_prepare(gcnn_ctx *c, bool capturing) {
   const size_t H = c->H, L = c->L, N = c->Nc;
   if (!c->f32_mem) {
     size_t off = 0;
@@ -557,7 +567,12 @@ int f32tc_prepare(gcnn_ctx *c) {
     const size_t o_p = take(4 * part), o_bad = take(4);
     char *m = nullptr;
     const cudaError_t e = cudaMalloc(&m, off);
-    if (e != cudaSuccess) return set_error(GCNN_ENOMEM, "cudaMalloc(%zu bytes): %s", off, cudaGetErrorString(e));
+    if (e == cudaErrorMemoryAllocation) {
+      (void)cudaGetLastError();
+      c->f32_off = true;
+      return GCNN_OK;
+    }
+    if (e != cudaSuccess) return set_error(GCNN_ECUDA, "cudaMalloc(%zu bytes): %s", off, cudaGetErrorString(e));
     // the planes' padding stays zero
     const cudaError_t z = cudaMemsetAsync(m, 0, off, c->stream);
     if (z != cudaSuccess) {
@@ -571,15 +586,17 @@ int f32tc_prepare(gcnn_ctx *c) {
     c->fwm = (float *)(m + o_fm); c->fwu = (float *)(m + o_fu);
     c->f32_part = (float *)(m + o_p); c->f32_part_floats = part;
     c->f32_bad = (unsigned *)(m + o_bad);
+    c->f32_bytes = off;
     c->dbytes += off;
     c->w3_stale = true;
   }
-  if (c->w3_stale) {
+  if (c->w3_stale || capturing) {
     LayerW w = layer_ptrs(c->params, c, 0);
     GCNN_CUDA_TRY(cudaMemsetAsync(c->f32_bad, 0, sizeof(unsigned), c->stream));
     GCNN_TRY(launch_slice_weights(c->H, 2 * c->H, c->L, w.msg_w, c->layer_size, c->wm3, c->fwm, c->f32_bad, c->stream));
     GCNN_TRY(launch_slice_weights(16 * c->H, c->H, c->L, w.upd_w, c->layer_size, c->wu3, c->fwu, c->f32_bad, c->stream));
-    c->w3_stale = false;
+    // a captured slicing has not run yet
+    if (!capturing) c->w3_stale = false;
   }
   return GCNN_OK;
 }

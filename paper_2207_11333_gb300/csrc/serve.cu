@@ -464,11 +464,32 @@ int gcnn_serve_create(const gcnn_ctx *model, const gcnn_serve_config *cfg, gcnn_
     if (rc != GCNN_OK) break;
     rc = gcnn_set_params(sl.ctx, model->params, sl.ctx->P, 1);
     if (rc != GCNN_OK) break;
-    // the slots' parameters never change: their slices are made once
-    if (f32tc_wanted(sl.ctx, max_nodes)) rc = f32tc_prepare(sl.ctx);
-    if (rc == GCNN_OK && cudaStreamSynchronize(sl.stream) != cudaSuccess)
-      rc = set_error(GCNN_ECUDA, "serve_create: cannot prepare a slot");
+  }
+  // the slots' parameters never change, so their slices for the tensor cores are
+  // made once; all slots or none, since a molecule's result may not depend on its
+  // slot, and none where they are more than a sixteenth of the memory that is left
+  // and the request pool would have to shrink for them
+  if (rc == GCNN_OK && f32tc_wanted(s->slots[0].ctx, max_nodes)) {
+    bool all = true;
+    size_t bytes = 0, free_b = 0, total_b = 0;
+    for (Slot &sl : s->slots) {
+      if (rc != GCNN_OK || !all) break;
+      rc = f32tc_prepare(sl.ctx);
+      all = rc == GCNN_OK && sl.ctx->f32_mem;
+      bytes += sl.ctx->f32_bytes;
+    }
+    if (rc == GCNN_OK && cudaMemGetInfo(&free_b, &total_b) != cudaSuccess)
+      rc = set_error(GCNN_ECUDA, "serve_create: cudaMemGetInfo");
+    if (bytes > free_b / 16 && cfg->queue_nodes > ((int64_t)(free_b / 2) - 2 * kMaxGraphEdges) / 9) all = false;
+    if (!all)
+      for (Slot &sl : s->slots) f32tc_release(sl.ctx);
+  }
+  for (Slot &sl : s->slots) {
     if (rc != GCNN_OK) break;
+    if (cudaStreamSynchronize(sl.stream) != cudaSuccess) {
+      rc = set_error(GCNN_ECUDA, "serve_create: cannot prepare a slot");
+      break;
+    }
     // every bucket's forward graph is captured now, so that no request
     // waits for a capture
     sl.exec.assign(cfg->n_buckets, nullptr);

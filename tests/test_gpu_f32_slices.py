@@ -81,6 +81,31 @@ def test_row_invariant_and_new_parameters(tmp_path):
     ctx.check()
 
 
+def test_captured_forward_follows_parameters(tmp_path):
+    """A capture made after an eager forward slices the weights anew in every replay."""
+    G = 110
+    gs, ost, st, _, params = _setup(tmp_path, G, 18, 22, 64, 2)
+    import paper_2207_11333_gb300 as g
+    with torch.cuda.stream(torch.cuda.Stream()):
+        ctx = g.Context(g.make_config(64, 2, G, gs.n_nodes, gs.n_edges, delta=st.delta()))
+        ctx.set_params(params)
+        b = ctx.collate(st, np.arange(G))
+        pred = torch.empty(G, device="cuda")
+        ctx.forward(b, pred, train=False)
+        graph = torch.cuda.CUDAGraph()
+        graph.capture_begin()
+        ctx.forward(b, pred, train=False)
+        graph.capture_end()
+        for p in (params, synth.init_params(23, 64, 2)):
+            ctx.set_params(p)
+            graph.replay()
+            torch.cuda.synchronize()
+            replayed = pred.cpu().numpy()
+            ctx.forward(b, pred, train=False)
+            ctx.check()
+            np.testing.assert_array_equal(replayed, pred.cpu().numpy())
+
+
 @pytest.mark.parametrize("bad", [float("inf"), float("-inf"), float("nan")])
 def test_non_finite_values(tmp_path, bad):
     """An infinite or undefined weight gives the plain path's activations: the

@@ -157,99 +157,127 @@ __device__ __forceinline__ void acc_sq(float4 &v, float4 m, float4 mean) {
 }
 
 // F32 / B16: whether the FP32 aggregates / the BF16 scaled operand are
-// written (one instantiation per output set keeps the other's code out)
-template <bool F32, bool B16, bool EDGE>
-__global__ void __launch_bounds__(kThreads, 8)
+// written (one instantiation per output set keeps the other's code out).
+// With LOOP a thread takes up to `items` of them, so that the next row's indices travel
+// while this one is reduced and stored: ncu showed 60% of the warps' time in
+// waits for the chain row_ptr -> sources -> Q rows.  Longer loops spread the
+// addresses that are written at one time: four items with the FP32 output alone
+// (300,000 atoms, H = 200: 331 -> 290 us; eight: 291), two with the BF16 operand,
+// whose 15 pieces a row write the most (64,400 atoms: 108 -> 106 us; four: 111,
+// eight: 122).  Registers: 64 as before for FP32 (72: 294 us, 80: 307), 72 with the
+// BF16 operand (64 spill: 122 us at eight items against 117).
+template <bool F32, bool B16, bool EDGE, bool LOOP>
+__global__ void __launch_bounds__(kThreads, LOOP && B16 ? 7 : 8)
 aggregate_fwd_kernel(int n_cap, int H, DevDims dims, const int *__restrict__ row_ptr,
                      const int *__restrict__ col, const float *__restrict__ PQ,
                      float *__restrict__ agg, float eps, unsigned *err, uint16_t *__restrict__ S16, int ld16,
-                     const float *__restrict__ amp, const float *__restrict__ att, Bonds bonds, int early) {
+                     const float *__restrict__ amp, const float *__restrict__ att, Bonds bonds, int early, int items) {
+  const int iters = LOOP ? items : 1;  // LOOP = false: one item a thread
   const int H4 = H >> 2;
-  const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  long long t = (long long)blockIdx.x * iters * kThreads + threadIdx.x;
   // the batch's sizes, the row's CSR range and its first sources (and the
   // degree scalers) come from the collator; with `early` they are read
   // before the dependency wait, overlapping the previous kernel's tail
+  long long work = 0;
   int N = 0, i = 0, c = 0, r0 = 0, r1 = 0;
   int j[kCache];
-  float s_amp = 0.f, s_att = 0.f;
-  auto load_row = [&]() {
-    N = min(n_cap, dims.nodes(n_cap));
-    if (t >= (long long)N * H4) return;
-    split_item(t, H4, i, c);
-    r0 = row_ptr[i];
-    r1 = row_ptr[i + 1];
+  auto load_sources = [&]() {
     if (r1 > r0 && r0 >= 0)
 #pragma unroll
       for (int k = 0; k < kCache; ++k) j[k] = col[min(r0 + k, r1 - 1)];
-    if (B16) {
-      s_amp = amp[i];
-      s_att = att[i];
-    }
+  };
+  auto load_row = [&]() {
+    N = min(n_cap, dims.nodes(n_cap));
+    work = (long long)N * H4;
+    if (t >= work) return;
+    split_item(t, H4, i, c);
+    r0 = row_ptr[i];
+    r1 = row_ptr[i + 1];
+    load_sources();
   };
   if (early) load_row();
   pdl_entry(GCNN_K_AGG_FWD);
   if (!early) load_row();
-  if (t >= (long long)N * H4) return;
-  const int d = r1 - r0;
-  float *out = F32 ? agg + (size_t)i * kAgg * H + c : nullptr;
+  const int di = kThreads / H4, dc = kThreads % H4 * 4;  // to the thread's next item
   const float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
-  if (d <= 0 || r0 < 0) {
-    if (d < 0 || r0 < 0) flag(err, kErrIndex);
-    if (F32)
+  for (int it = 0; it < iters && t < work; ++it) {
+    // the next item's row range is in flight during this one's arithmetic, its
+    // sources during this one's stores
+    t += kThreads;
+    const bool more = it + 1 < iters && t < work;
+    const int ic = i, cc = c, d = r1 - r0;
+    i += di;
+    c += dc;
+    if (c >= H) {
+      c -= H;
+      ++i;
+    }
+    int n0 = 0, n1 = 0;
+    if (more) {
+      n0 = row_ptr[i];
+      n1 = row_ptr[i + 1];
+    }
+    float s_amp = 0.f, s_att = 0.f;
+    if (B16 && d > 0) {
+      s_amp = amp[ic];
+      s_att = att[ic];
+    }
+    float4 s = z, mean = z, mn = z, mx = z, sd = z;
+    if (d <= 0 || r0 < 0) {
+      if (d < 0 || r0 < 0) flag(err, kErrIndex);
+    } else {
+      // every load of the row is issued before the arithmetic: the first kCache
+      // sources (indices clamped into the row, so short rows repeat their last
+      // edge and use only the first d; read above), then P and the gathered Q rows
+      const float4 P = ld4(PQ + (size_t)ic * 2 * H + cc);
+      float4 mc[kCache];
+      if (gather_first<EDGE>(PQ, j, ic, N, H, cc, P, mc, bonds, r0, r1)) flag(err, kErrIndex);
+      mn = make_float4(FLT_MAX, FLT_MAX, FLT_MAX, FLT_MAX);
+      mx = make_float4(-FLT_MAX, -FLT_MAX, -FLT_MAX, -FLT_MAX);
+      auto take = [&](float4 m) {
+        s = add4(s, m);
+        mn.x = fminf(mn.x, m.x); mn.y = fminf(mn.y, m.y); mn.z = fminf(mn.z, m.z); mn.w = fminf(mn.w, m.w);
+        mx.x = fmaxf(mx.x, m.x); mx.y = fmaxf(mx.y, m.y); mx.z = fmaxf(mx.z, m.z); mx.w = fmaxf(mx.w, m.w);
+      };
 #pragma unroll
-      for (int a = 0; a < kAgg; ++a) st4(out + a * H, z);
-    if (B16)
-      for (int a = 0; a < kScalers * kAgg; ++a) st_bf16x4(S16 + (size_t)i * ld16 + a * H + c, 0.f, 0.f, 0.f, 0.f);
-    return;
-  }
-  // every load of the row is issued before the arithmetic: the first kCache
-  // sources (indices clamped into the row, so short rows repeat their last
-  // edge and use only the first d; read above), then P and the gathered Q rows
-  const float4 P = ld4(PQ + (size_t)i * 2 * H + c);
-  float4 mc[kCache];
-  if (gather_first<EDGE>(PQ, j, i, N, H, c, P, mc, bonds, r0, r1)) flag(err, kErrIndex);
-  float4 s = z;
-  float4 mn = make_float4(FLT_MAX, FLT_MAX, FLT_MAX, FLT_MAX);
-  float4 mx = make_float4(-FLT_MAX, -FLT_MAX, -FLT_MAX, -FLT_MAX);
-  auto take = [&](float4 m) {
-    s = add4(s, m);
-    mn.x = fminf(mn.x, m.x); mn.y = fminf(mn.y, m.y); mn.z = fminf(mn.z, m.z); mn.w = fminf(mn.w, m.w);
-    mx.x = fmaxf(mx.x, m.x); mx.y = fmaxf(mx.y, m.y); mx.z = fmaxf(mx.z, m.z); mx.w = fmaxf(mx.w, m.w);
-  };
+      for (int k = 0; k < kCache; ++k)
+        if (k < d) take(mc[k]);
+      for (int e = r0 + kCache; e < r1; ++e) take(message<EDGE>(PQ, source(col, e, N, err), H, cc, P, bonds, e));
+      const float df = (float)d;
+      mean = div_count(s, df);
+      float4 v = z;  // two-pass variance
 #pragma unroll
-  for (int k = 0; k < kCache; ++k)
-    if (k < d) take(mc[k]);
-  for (int e = r0 + kCache; e < r1; ++e) take(message<EDGE>(PQ, source(col, e, N, err), H, c, P, bonds, e));
-  const float df = (float)d;
-  const float4 mean = div_count(s, df);
-  float4 v = z;  // two-pass variance
+      for (int k = 0; k < kCache; ++k)
+        if (k < d) acc_sq(v, mc[k], mean);
+      for (int e = r0 + kCache; e < r1; ++e)
+        acc_sq(v, message<EDGE>(PQ, source(col, e, N, err), H, cc, P, bonds, e), mean);
+      v = div_count(v, df);
+      sd.x = sqrtf(fmaxf(v.x, 0.f) + eps);
+      sd.y = sqrtf(fmaxf(v.y, 0.f) + eps);
+      sd.z = sqrtf(fmaxf(v.z, 0.f) + eps);
+      sd.w = sqrtf(fmaxf(v.w, 0.f) + eps);
+    }
+    r0 = n0;
+    r1 = n1;
+    load_sources();
+    if (F32) {
+      float *out = agg + (size_t)ic * kAgg * H + cc;
+      st4(out + 0 * H, s);
+      st4(out + 1 * H, mean);
+      st4(out + 2 * H, mn);
+      st4(out + 3 * H, mx);
+      st4(out + 4 * H, sd);
+    }
+    if (B16) {  // scaler-major: identity, amplification, attenuation
+      const float4 vv[kAgg] = {s, mean, mn, mx, sd};
+      const float sc[kScalers] = {1.f, s_amp, s_att};
+      uint16_t *o = S16 + (size_t)ic * ld16 + cc;
 #pragma unroll
-  for (int k = 0; k < kCache; ++k)
-    if (k < d) acc_sq(v, mc[k], mean);
-  for (int e = r0 + kCache; e < r1; ++e)
-    acc_sq(v, message<EDGE>(PQ, source(col, e, N, err), H, c, P, bonds, e), mean);
-  v = div_count(v, df);
-  float4 sd;
-  sd.x = sqrtf(fmaxf(v.x, 0.f) + eps);
-  sd.y = sqrtf(fmaxf(v.y, 0.f) + eps);
-  sd.z = sqrtf(fmaxf(v.z, 0.f) + eps);
-  sd.w = sqrtf(fmaxf(v.w, 0.f) + eps);
-  if (F32) {
-    st4(out + 0 * H, s);
-    st4(out + 1 * H, mean);
-    st4(out + 2 * H, mn);
-    st4(out + 3 * H, mx);
-    st4(out + 4 * H, sd);
-  }
-  if (B16) {  // scaler-major: identity, amplification, attenuation
-    const float4 vv[kAgg] = {s, mean, mn, mx, sd};
-    const float sc[kScalers] = {1.f, s_amp, s_att};
-    uint16_t *o = S16 + (size_t)i * ld16 + c;
+      for (int q = 0; q < kScalers; ++q)
 #pragma unroll
-    for (int q = 0; q < kScalers; ++q)
-#pragma unroll
-      for (int a = 0; a < kAgg; ++a)
-        st_bf16x4(o + (q * kAgg + a) * H, sc[q] * vv[a].x, sc[q] * vv[a].y, sc[q] * vv[a].z, sc[q] * vv[a].w);
+        for (int a = 0; a < kAgg; ++a)
+          st_bf16x4(o + (q * kAgg + a) * H, sc[q] * vv[a].x, sc[q] * vv[a].y, sc[q] * vv[a].z, sc[q] * vv[a].w);
+    }
   }
 }
 
@@ -736,14 +764,21 @@ int launch_aggregate_fwd(int n_nodes, int H, DevDims dims, const int *row_ptr, c
   if (n_nodes <= 0) return GCNN_OK;
   const long long work = (long long)n_nodes * (H / 4);
   using K = void (*)(int, int, DevDims, const int *, const int *, const float *, float *, float, unsigned *,
-                     uint16_t *, int, const float *, const float *, Bonds, int);
-  static const K table[8] = {aggregate_fwd_kernel<false, false, false>, aggregate_fwd_kernel<false, true, false>,
-                             aggregate_fwd_kernel<true, false, false>,  aggregate_fwd_kernel<true, true, false>,
-                             aggregate_fwd_kernel<false, false, true>,  aggregate_fwd_kernel<false, true, true>,
-                             aggregate_fwd_kernel<true, false, true>,   aggregate_fwd_kernel<true, true, true>};
-  const K kernel = table[(F > 0 ? 4 : 0) + (agg ? 2 : 0) + (S16 ? 1 : 0)];
-  GCNN_TRY(launch(kernel, ceil_div(work, kThreads), kThreads, 0, s, n_nodes, H, dims, row_ptr, col, PQ, agg, eps, err,
-                  S16, ld16, amp, att, Bonds{eattr, wE, F}, idx_early ? 1 : 0));
+                     uint16_t *, int, const float *, const float *, Bonds, int, int);
+  // with bond features one item a thread: their sums leave no registers for the next row
+  static const K table[12] = {
+      aggregate_fwd_kernel<false, false, false, false>, aggregate_fwd_kernel<false, true, false, false>,
+      aggregate_fwd_kernel<true, false, false, false>,  aggregate_fwd_kernel<true, true, false, false>,
+      aggregate_fwd_kernel<false, false, false, true>,  aggregate_fwd_kernel<false, true, false, true>,
+      aggregate_fwd_kernel<true, false, false, true>,   aggregate_fwd_kernel<true, true, false, true>,
+      aggregate_fwd_kernel<false, false, true, false>,  aggregate_fwd_kernel<false, true, true, false>,
+      aggregate_fwd_kernel<true, false, true, false>,   aggregate_fwd_kernel<true, true, true, false>};
+  // several items a thread only where 16 blocks per SM remain
+  const long long most = work / (16LL * kThreads * num_sms());
+  const int iters = F > 0 ? 1 : (int)std::max(1LL, std::min(S16 ? 2LL : 4LL, most));
+  const K kernel = table[(F > 0 ? 8 : iters > 1 ? 4 : 0) + (agg ? 2 : 0) + (S16 ? 1 : 0)];
+  GCNN_TRY(launch(kernel, ceil_div(work, (long long)kThreads * iters), kThreads, 0, s, n_nodes, H, dims, row_ptr, col,
+                  PQ, agg, eps, err, S16, ld16, amp, att, Bonds{eattr, wE, F}, idx_early ? 1 : 0, iters));
   return GCNN_OK;
 }
 

@@ -35,7 +35,7 @@ __global__ void embed_kernel(int n_cap, int H, DevDims dims, const uint8_t *__re
 constexpr int kMaxTypes = 16;
 constexpr int kRedThreads = 256;
 constexpr int kEmbBwdThreads = 512;   // one block per 4-column slice: nodes strided over the block
-constexpr int kColsumThreads = 1024;
+constexpr int kColsumThreads = 256;
 constexpr int kColsumWidth = 32;    // columns per CTA of the bias sums
 constexpr int kColsumMaxRanks = 8;  // CTAs of a cluster (row ranges), portable size
 
@@ -826,8 +826,13 @@ adam_kernel(AdamSpan sp, int advance, float *__restrict__ p, const float *__rest
 // row's 128 bytes, so a warp covers four rows per load.  The rows are cut into
 // gridDim.y contiguous ranges, one per CTA of a cluster.  Fixed order
 // throughout: each thread adds its rows in increasing order, the four rows of
-// a warp by butterfly, the warps in index order, and the cluster's CTAs in
+// a warp by butterfly, sums and warps in index order, and the cluster's CTAs in
 // rank order (distributed shared memory), so the sums are bit-reproducible.
+// CTAs of 256 threads with eight loads in flight each, since the sums run beside
+// the data-gradient chain in the overlapped backward and a CTA of 1,024 threads
+// (whole registers of an SM) held it up: the training step of 128 molecules,
+// H = 200, 390 -> 380 us, of 13 molecules 265 -> 260 us; alone 18,000 atoms take
+// the same 15 us (four loads in flight: 37 us; 512 threads with four: 26 us).
 // The launch makes the cluster (1, gridDim.y, 1), so a CTA's rank in its
 // cluster is blockIdx.y and rank 0 writes the group's sums.
 __global__ void __launch_bounds__(kColsumThreads)
@@ -835,8 +840,11 @@ colsum_kernel(int n_cap, int cols0, int cols, DevDims dims, const float *__restr
               const float *__restrict__ mask, int ldm, const float *__restrict__ a1, int ld1,
               float *__restrict__ out0, float *__restrict__ out1) {
   pdl_entry(GCNN_K_COLSUM);
-  constexpr int kWarps = kColsumThreads / 32, kRowsPerPass = kColsumThreads / 8;
-  __shared__ float4 sh[kWarps][8];
+  // kSums sums a thread: the rows of a CTA in blocks of 128, sum k takes the k-th part
+  // of every block
+  constexpr int kWarps = kColsumThreads / 32, kRows = kColsumThreads / 8, kSums = 128 / kRows, kLoads = 8;
+  static_assert(kLoads % kSums == 0, "a load belongs to one sum in every pass");
+  __shared__ float4 sh[kWarps * kSums][8];
   __shared__ float4 part[8];
   const int N = min(n_cap, dims.nodes(n_cap));
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, q = lane & 7;
@@ -844,46 +852,51 @@ colsum_kernel(int n_cap, int cols0, int cols, DevDims dims, const float *__restr
   const bool first = c < cols0;
   const int seg = (N + (int)gridDim.y - 1) / (int)gridDim.y;
   const int i0 = (int)blockIdx.y * seg, i1 = min(N, i0 + seg);
-  float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+  float4 acc[kSums];
+#pragma unroll
+  for (int k = 0; k < kSums; ++k) acc[k] = make_float4(0.f, 0.f, 0.f, 0.f);
   if (c < cols) {
     const float *src = first ? a0 + c : a1 + (c - cols0);
     const int ld = first ? ld0 : ld1;
     const float *mk = first ? mask : nullptr;
     // every load of a pass before any use: rows past the range repeat its
     // last one and are not added
-    for (int i = i0 + (threadIdx.x >> 3); i < i1; i += 4 * kRowsPerPass) {
-      float4 x[4], m[4];
+    for (int i = i0 + (threadIdx.x >> 3); i < i1; i += kLoads * kRows) {
+      float4 x[kLoads], m[kLoads];
 #pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        const size_t r = (size_t)min(i + u * kRowsPerPass, i1 - 1);
+      for (int u = 0; u < kLoads; ++u) {
+        const size_t r = (size_t)min(i + u * kRows, i1 - 1);
         x[u] = ld4(src + r * ld);
         if (mk) m[u] = ld4(mk + r * ldm + c);
       }
 #pragma unroll
-      for (int u = 0; u < 4; ++u) {
+      for (int u = 0; u < kLoads; ++u) {
         if (mk) {
           x[u].x = m[u].x > 0.f ? x[u].x : 0.f;
           x[u].y = m[u].y > 0.f ? x[u].y : 0.f;
           x[u].z = m[u].z > 0.f ? x[u].z : 0.f;
           x[u].w = m[u].w > 0.f ? x[u].w : 0.f;
         }
-        if (i + u * kRowsPerPass < i1) acc = add4(acc, x[u]);
+        if (i + u * kRows < i1) acc[u % kSums] = add4(acc[u % kSums], x[u]);
       }
     }
   }
 #pragma unroll
-  for (int o = 8; o < 32; o <<= 1) {
-    acc.x += __shfl_xor_sync(0xffffffffu, acc.x, o);
-    acc.y += __shfl_xor_sync(0xffffffffu, acc.y, o);
-    acc.z += __shfl_xor_sync(0xffffffffu, acc.z, o);
-    acc.w += __shfl_xor_sync(0xffffffffu, acc.w, o);
+  for (int k = 0; k < kSums; ++k) {
+#pragma unroll
+    for (int o = 8; o < 32; o <<= 1) {
+      acc[k].x += __shfl_xor_sync(0xffffffffu, acc[k].x, o);
+      acc[k].y += __shfl_xor_sync(0xffffffffu, acc[k].y, o);
+      acc[k].z += __shfl_xor_sync(0xffffffffu, acc[k].z, o);
+      acc[k].w += __shfl_xor_sync(0xffffffffu, acc[k].w, o);
+    }
+    if (lane < 8) sh[k * kWarps + w][lane] = acc[k];
   }
-  if (lane < 8) sh[w][lane] = acc;
   __syncthreads();
   if (threadIdx.x < 8) {
     float4 sum = sh[0][threadIdx.x];
 #pragma unroll
-    for (int k = 1; k < kWarps; ++k) sum = add4(sum, sh[k][threadIdx.x]);
+    for (int k = 1; k < kWarps * kSums; ++k) sum = add4(sum, sh[k][threadIdx.x]);
     part[threadIdx.x] = sum;
   }
   colsum_cluster_sync();

@@ -77,10 +77,15 @@ extern "C" {
 #define GCNN_EAGAIN (-7)    /* result not ready / queue full: call again      */
 #define GCNN_ESTATE (-8)    /* call out of order (e.g. backward w/o forward)  */
 
-#define GCNN_PREC_FP32 0    /* FP32 everywhere (SIMT FFMA GEMMs)              */
+/* FP32 everywhere: FFMA GEMMs; inference forwards without bond features and
+ * with 64 <= hidden <= 256 (from 2,048 nodes, or row-invariant) take exact
+ * integer slices of the FP32 values through the tensor cores instead, with an
+ * error at or below the FFMA products'. */
+#define GCNN_PREC_FP32 0
 #define GCNN_PREC_BF16 1    /* BF16 tensor-core GEMMs, FP32 accumulate        */
 
-/* Row-invariant arithmetic: no split-K in the GEMMs, so each node's and each
+/* Row-invariant arithmetic: no split-K in the BF16 GEMMs and fixed K chunks in
+ * the FP32 ones, so each node's and each
  * graph's results depend only on its own graph, never on its batch-mates
  * (bit-identical alone and in any batch).  Used by the inference server. */
 #define GCNN_FLAG_ROW_INVARIANT 1
@@ -371,7 +376,10 @@ int gcnn_profile_enable(gcnn_ctx *ctx, int enable);
  * resets the counters. */
 int gcnn_profile_read(gcnn_ctx *ctx, double *ms, int64_t *launches);
 /* Device bytes held by the context (parameters, optimiser state, batch,
- * activations and workspace; one allocation made by gcnn_create). */
+ * activations and workspace): one allocation made by gcnn_create, plus the
+ * tensor-core slices' buffers from the first FP32 inference forward that takes
+ * them (without room for them it runs on the CUDA cores, as a capture by the
+ * caller does that comes before them). */
 int gcnn_memory(const gcnn_ctx *ctx, int64_t *arena_bytes);
 /* Kernels in the CUDA graph of the most recent gcnn_train_step or
  * gcnn_train_step_range (0 if it ran eagerly; the latter's count includes its

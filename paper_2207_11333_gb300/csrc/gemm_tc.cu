@@ -45,12 +45,11 @@ constexpr int BM = 128, BK = 64, STAGES = 3, kThreads = 256;
 constexpr int kLongStages = 6, kLongTiles = 64;
 constexpr int kMaxBN = 128;
 // Co-resident CTAs per SM: about 100 KB of shared memory and at most 128
-// registers per thread each.  One CTA issues its MMAs at a latency-bound rate
-// well below the SM's tensor throughput for tiles up to 128 wide; a second
-// CTA on the same SM, from another stream's GEMM or from the next wave of a
-// large grid, nearly doubles the SM's rate.  A launch is planned for at most
-// one CTA per SM: within one short launch a second CTA per SM only adds its
-// fixed costs (measured).
+// registers per thread each.  A CTA's main loop waits for operands (an SM takes
+// in 90-100 GB/s while all load) and its fixed costs leave the tensor core idle;
+// a second CTA on the same SM, from another stream's GEMM, uses that time.  A
+// launch is planned for at most one CTA per SM: within one short launch a
+// second CTA per SM only adds its fixed costs (measured).
 constexpr int kCtasPerSm = 2;
 constexpr int kDrain = 4;  // 8-column TMEM loads in flight per thread in the epilogue (register budget)
 constexpr int kATileBytes = BM * BK * 2;        // 16 KB
